@@ -25,6 +25,7 @@ SOURCES = [
     "runtime.cu",
     "rows_f32.cu",
     "rows_f16.cu",
+    "rows_f16_inv.cu",
     "rows_fp8.cu",
     "sar_nn.cu",
     "sar_nt.cu",

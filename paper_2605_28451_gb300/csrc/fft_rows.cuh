@@ -61,6 +61,7 @@ struct RowArgs {
   const float2* tw;        // W_N^i for i in [0, N), FP32
   const float2* h;         // filter spectrum [N] (compress only)
   long long h_stride;      // compress: points between the filters of consecutive lines (0: one filter for all)
+  int h_prefetch;          // compress: every line has its own filter, in device memory: prefetch it into L2
   long long lines;         // number of lines
   long long in_stride;     // points between consecutive input lines
   long long out_stride;    // points between consecutive output lines
@@ -68,6 +69,7 @@ struct RowArgs {
   float out_scale;         // applied before the final rounding (FP8 block exponent)
   int* status;             // device status word (bounded waits record timeouts here)
   int variant;             // RowVariant
+  const float4* tw_wide;   // lines of 512 .. 16384 points: twiddle table of wide_rows.cuh, or null
   const float2* tw_line;   // N >= 8192: pass-major table of the 4096-point row transforms
   const float2* tw_4step;  // N >= 8192: four-step twiddles T[k1][n2] = W_N^{n2 k1}
   const void* tc_b;        // tensor-core variant: 16-point DFT matrix, real form, FP16 [32][32]
@@ -1226,6 +1228,12 @@ cudaError_t launch_rows_plain_x(const RowArgs& a, cudaStream_t stream, bool l2_p
   return cudaGetLastError();
 }
 
+}  // namespace bfp
+
+#include "wide_rows.cuh"   // the kernels with 32 or 64 points per thread, built on the definitions above
+
+namespace bfp {
+
 template <int N, class TIn, class TOut, int MODE, bool NAIVE, bool SCALED, bool TLOAD = false,
           bool TSTORE = false>
 cudaError_t launch_rows_n(const RowArgs& a, cudaStream_t stream) {
@@ -1250,6 +1258,13 @@ cudaError_t launch_rows_n(const RowArgs& a, cudaStream_t stream) {
     return launch_cluster_n<N, TIn, TOut, MODE, NAIVE, SCALED>(a, stream);
   } else {
   using S = RowShape<N, TLOAD || TSTORE>;
+  if constexpr (!TLOAD && !TSTORE && !NAIVE && N >= 512) {
+    if constexpr (kWideOffered<N, TIn, MODE>) {
+      if ((a.variant == kRowsPlain4L2 || a.variant == kRowsPlain4) && a.tw_wide != nullptr &&
+          a.lines >= kWideMinLines<N>)
+        return launch_wide_n<N, TIn, TOut, MODE, SCALED>(a, stream, a.variant == kRowsPlain4L2);
+    }
+  }
   // Exchange variants for dense forward / inverse rows (FP16 exchange only
   // for FP16 storage): see RowVariant.
   if constexpr (!TLOAD && !TSTORE && !SCALED && MODE != kCompress && N >= 256 && N <= 4096 &&
@@ -1258,9 +1273,7 @@ cudaError_t launch_rows_n(const RowArgs& a, cudaStream_t stream) {
       constexpr bool kHalf = std::is_same<TIn, __half2>::value;
       switch (a.variant) {
         case kRowsPlainPP: return launch_rows_plain_x<N, TIn, TOut, MODE, NAIVE, kXchF32PP>(a, stream);
-        case kRowsPlain4: return launch_rows_plain_x<N, TIn, TOut, MODE, NAIVE, kXchF32, 4>(a, stream);
         case kRowsPlainL2: return launch_rows_plain_x<N, TIn, TOut, MODE, NAIVE, kXchF32>(a, stream, true);
-        case kRowsPlain4L2: return launch_rows_plain_x<N, TIn, TOut, MODE, NAIVE, kXchF32, 4>(a, stream, true);
         case kRowsTmaPP: return launch_rows_tma_n<N, TIn, TOut, MODE, NAIVE, SCALED, kXchF32PP>(a, stream);
         case kRowsPlainH:
           if constexpr (kHalf) return launch_rows_plain_x<N, TIn, TOut, MODE, NAIVE, kXchF16>(a, stream);

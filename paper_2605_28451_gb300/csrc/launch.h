@@ -7,13 +7,11 @@
 
 namespace bfp {
 
-// float2 -> float2 rows: mode in {kForward, kInverse, kCompress}.
+// float2 -> float2 rows: mode in {kForward, kInverse}.
 cudaError_t launch_rows_f32(int log2n, int mode, const RowArgs& a, cudaStream_t s);
 // __half2 -> __half2 rows; naive selects the unshifted inverse (Section III-B).
 cudaError_t launch_rows_f16(int log2n, int mode, bool naive, const RowArgs& a, cudaStream_t s);
-// Mixed-storage compress: float2 raw -> __half2 out, or __half2 raw -> float2 out.
-cudaError_t launch_compress_c64_to_f16(int log2n, bool naive, const RowArgs& a, cudaStream_t s);
-cudaError_t launch_compress_f16_to_c64(int log2n, const RowArgs& a, cudaStream_t s);
+cudaError_t launch_rows_f16_inverse(int log2n, bool naive, const RowArgs& a, cudaStream_t s);
 // FP8 rows (fmt 0 = E4M3, 1 = E5M2); mode in {kForward, kInverse}.
 cudaError_t launch_rows_fp8(int log2n, int mode, int fmt, const RowArgs& a, cudaStream_t s);
 

@@ -146,10 +146,43 @@ __global__ void twopass_twiddle_kernel(float2* tw, int n) {
   tw[i] = make_float2(float(c), float(s));
 }
 
+// Table of the 32- / 64-point-per-thread kernels (wide_rows.cuh): the pass
+// with sub-length ns and radix r holds W_{ns r}^{k q}, q < r, at entry
+// (ns == first ? 0 : ns) + 2 ((q / 2) ns + k) + (q & 1).  FP64 sincospi, rounded
+// once to FP32.
+__global__ void wide_twiddle_kernel(float2* tw, int ns, int radix, int off) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= ns * radix) return;
+  const int k = i % ns, q = i / ns;
+  double s, c;
+  sincospi(-2.0 * double((long long)k * q) / (double(ns) * double(radix)), &s, &c);
+  tw[off + 2 * ((q / 2) * ns + k) + (q & 1)] = make_float2(float(c), float(s));
+}
+
+// The passes of a line of 2^log2n points: first radix (= points per thread)
+// and the radices after it (0: none).
+struct WidePlan {
+  int first, second, third;
+};
+template <int N> constexpr WidePlan wide_plan_of() {
+  constexpr int p = bfp::WideShape<N>::P, r2 = bfp::wide_radix<N>(p), r3 = N / (p * r2);
+  return {p, r2, r3 > 1 ? r3 : 0};
+}
+WidePlan wide_plan(int log2n) {
+  switch (log2n) {
+    case 9: return wide_plan_of<512>();
+    case 10: return wide_plan_of<1024>();
+    case 11: return wide_plan_of<2048>();
+    case 12: return wide_plan_of<4096>();
+    case 13: return wide_plan_of<8192>();
+    default: return wide_plan_of<16384>();
+  }
+}
+
 // Per-device, per-length twiddle tables, created on first use and kept for
 // the life of the process (a few hundred KB per device at most).  Keys
 // 0..16: pass-major Stockham tables; 100 + log2 n: four-step tables;
-// 500 + log2 n: two-pass tables.
+// 500 + log2 n: two-pass tables; 600 + log2 n: wide_rows.cuh's tables.
 std::mutex g_tw_mutex;
 std::map<std::pair<int, int>, float2*> g_tw;
 
@@ -165,13 +198,19 @@ int get_twiddles(int log2n, float2** out) {
     return BFPFFT_OK;
   }
   if (fault("alloc")) return BFPFFT_ERR_OOM;
-  const bool two = log2n >= 500;
-  const bool four = !two && log2n >= 100;
-  const int n = 1 << (two ? log2n - 500 : four ? log2n - 100 : log2n);
+  const bool wide = log2n >= 600;
+  const bool two = !wide && log2n >= 500;
+  const bool four = !wide && !two && log2n >= 100;
+  const int n = 1 << (wide ? log2n - 600 : two ? log2n - 500 : four ? log2n - 100 : log2n);
   float2* tw = nullptr;
-  e = cudaMalloc(&tw, sizeof(float2) * n);
+  const WidePlan wp = wide ? wide_plan(log2n - 600) : WidePlan{0, 0, 0};
+  const int second = wp.first * wp.second;   // entries of the second pass (all of them, or the third's offset)
+  e = cudaMalloc(&tw, sizeof(float2) * size_t(wide && wp.third ? n + second : n));
   if (e != cudaSuccess) return cuda_status(e);
-  if (two) {
+  if (wide) {
+    wide_twiddle_kernel<<<(second + 255) / 256, 256>>>(tw, wp.first, wp.second, 0);
+    if (wp.third) wide_twiddle_kernel<<<(n + 255) / 256, 256>>>(tw, second, wp.third, second);
+  } else if (two) {
     twopass_twiddle_kernel<<<(n + 255) / 256, 256>>>(tw, n);
   } else if (four) {
     fourstep_twiddle_kernel<<<(n + 255) / 256, 256>>>(tw, n);
@@ -344,14 +383,21 @@ int get_tc_matrix(void** out) {
   return BFPFFT_OK;
 }
 
-// Lines of 8192 points and more use the four-step kernel: the 4096-point
-// row table and the four-step table of their length.
-int fourstep_tables(int log2n, bfp::RowArgs* a) {
+// Tables of the kernels that go by the length: wide_rows.cuh's for 512 ..
+// 16384 points; the 4096-point row table and the four-step table of their
+// length for the four-step kernel's 8192 points and more.
+int length_tables(int log2n, bfp::RowArgs* a) {
   a->tw_line = nullptr;
   a->tw_4step = nullptr;
-  if (log2n < 13) return BFPFFT_OK;
+  a->tw_wide = nullptr;
   float2* t = nullptr;
-  int st = get_twiddles(12, &t);
+  int st = BFPFFT_OK;
+  if (log2n >= bfp::kWideMinLog2 && log2n <= bfp::kWideMaxLog2) {
+    if ((st = get_twiddles(600 + log2n, &t)) != BFPFFT_OK) return st;
+    a->tw_wide = reinterpret_cast<const float4*>(t);
+  }
+  if (log2n < 13) return BFPFFT_OK;
+  st = get_twiddles(12, &t);
   if (st != BFPFFT_OK) return st;
   a->tw_line = t;
   st = get_twiddles(100 + log2n, &t);
@@ -370,7 +416,7 @@ int row_args(int log2n, bfp::RowArgs* a) {
   a->in_scale = 1.f;
   a->out_scale = 1.f;
   a->variant = rows_variant();
-  return fourstep_tables(log2n, a);
+  return length_tables(log2n, a);
 }
 
 bool valid_dtype(int d) { return d >= BFPFFT_F32 && d <= BFPFFT_BF16; }
@@ -405,7 +451,10 @@ struct bfpfft_plan_s {
   int dtype;
   int direction;
   int device;
-  float2* tw;          // shared table from the per-device cache (not owned)
+  float2* tw;          // shared tables from the per-device cache (not owned): RowArgs' fields
+  const float4* tw_wide = nullptr;
+  const float2* tw_line = nullptr;
+  const float2* tw_4step = nullptr;
   int* status;         // the plan's own device status word (owned): timeouts, non-finite outputs
   int flags = 0;       // BFPFFT_CHECK_FINITE
   int arith = 0;       // enum bfpfft_arith: the arithmetic the transforms run in
@@ -580,7 +629,7 @@ static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStre
     const float sc = float(1 << ((l + 1) / 2));       // FP8 block exponent of a uniform plan of this length
     a.in_scale = plan->kind >= 2 && mode == bfp::kInverse ? sc : 1.f;
     a.out_scale = plan->kind >= 2 && mode == bfp::kForward ? 1.f / sc : 1.f;
-    result = fourstep_tables(l, &a);
+    result = length_tables(l, &a);
     if (result != BFPFFT_OK) break;
     cudaError_t e;
     switch (plan->kind) {
@@ -947,12 +996,17 @@ int bfpfft_plan_create(bfpfft_plan* out, int64_t n, int64_t batch, int dtype, in
   }
   cudaError_t e = cudaGetDevice(&p->device);
   int st = e == cudaSuccess ? get_twiddles(l, &p->tw) : cuda_status(e);
+  bfp::RowArgs tables{};
+  if (st == BFPFFT_OK) st = length_tables(l, &tables);   // now, not inside a capture
   if (st == BFPFFT_OK) st = alloc_plan_status(&p->status);
   if (st != BFPFFT_OK) {
     free_plan_resources(p);
     delete p;
     return st;
   }
+  p->tw_wide = tables.tw_wide;
+  p->tw_line = tables.tw_line;
+  p->tw_4step = tables.tw_4step;
   tune_on_create(p);
   *out = p;
   return BFPFFT_OK;
@@ -1031,9 +1085,10 @@ int bfpfft_plan_create_many(bfpfft_plan* out, int64_t count, const int64_t* n, c
     st = get_twiddles(l, &t);
     tw_host[l] = t;
     p->tw_len[l] = t;
-    if (st == BFPFFT_OK && l >= 13) {
-      bfp::RowArgs tmp{};
-      st = fourstep_tables(l, &tmp);
+    if (st != BFPFFT_OK) break;
+    bfp::RowArgs tmp{};
+    st = length_tables(l, &tmp);
+    if (l >= 13) {
       tw_host[12] = tmp.tw_line;
       tw4_host[l] = tmp.tw_4step;
     }
@@ -1127,10 +1182,9 @@ int bfpfft_exec(bfpfft_plan plan, const void* in, void* out, void* stream) {
     const int stc = get_tc_matrix(const_cast<void**>(&a.tc_b));
     if (stc != BFPFFT_OK) return stc;
   }
-  {
-    const int st4 = fourstep_tables(plan->log2n, &a);
-    if (st4 != BFPFFT_OK) return st4;
-  }
+  a.tw_wide = plan->tw_wide;
+  a.tw_line = plan->tw_line;
+  a.tw_4step = plan->tw_4step;
   a.lines = plan->batch;
   a.in_stride = plan->n;
   a.out_stride = plan->n;
@@ -1367,6 +1421,7 @@ int bfp_spectral_filter(const void* x, int x_dtype, const void* h, int64_t h_str
   a.out = out;
   a.h = static_cast<const float2*>(h);
   a.h_stride = h_stride;
+  a.h_prefetch = h_stride != 0 && device_memory(h);
   if (!device_memory(x)) {
     a.variant = without_l2(a.variant);
     a.no_prefetch = 1;
