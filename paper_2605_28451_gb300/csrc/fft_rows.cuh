@@ -70,6 +70,8 @@ struct RowArgs {
   int* status;             // device status word (bounded waits record timeouts here)
   int variant;             // RowVariant
   const float4* tw_wide;   // lines of 512 .. 16384 points: twiddle table of wide_rows.cuh, or null
+  const float4* tw_long;   // lines of 32768 / 65536 points: column-to-row twiddles of long_rows.cuh, or null
+  const float4* tw_row1024;   // ... and wide_rows.cuh's layout of its 1024 = 64 x 16 rows
   const float2* tw_line;   // N >= 8192: pass-major table of the 4096-point row transforms
   const float2* tw_4step;  // N >= 8192: four-step twiddles T[k1][n2] = W_N^{n2 k1}
   const void* tc_b;        // tensor-core variant: 16-point DFT matrix, real form, FP16 [32][32]
@@ -1230,15 +1232,17 @@ cudaError_t launch_rows_plain_x(const RowArgs& a, cudaStream_t stream, bool l2_p
 
 }  // namespace bfp
 
-#include "wide_rows.cuh"   // the kernels with 32 or 64 points per thread, built on the definitions above
+// Kernels with 32 or 64 points per thread, built on the definitions above.
+#include "long_rows.cuh"
+#include "wide_rows.cuh"
 
 namespace bfp {
 
 template <int N, class TIn, class TOut, int MODE, bool NAIVE, bool SCALED, bool TLOAD = false,
           bool TSTORE = false>
 cudaError_t launch_rows_n(const RowArgs& a, cudaStream_t stream) {
-  // Dense lines of 32768 and 65536 points: the four-step kernel over a
-  // cluster.  Lines of 8192 and 16384 points run on one CTA of N / 16 threads
+  // Dense lines of 32768 and 65536 points: a cluster per line (long_rows.cuh,
+  // or the four-step kernel for a few lines).  Lines of 8192 and 16384 points run on one CTA of N / 16 threads
   // (512 at 2 CTAs per SM, or 1024), which measured 1.4x faster than the
   // four-step kernel for plain transforms and 3x faster than the per-pass
   // cluster kernel for compression; longer lines the four-step kernel does not
@@ -1246,11 +1250,14 @@ cudaError_t launch_rows_n(const RowArgs& a, cudaStream_t stream) {
   // cluster kernel.
   if constexpr (!TLOAD && !TSTORE && N >= 32768) {
     if constexpr (MODE != kCompress && !NAIVE && std::is_same<TIn, TOut>::value) {
-      if (a.tw_4step != nullptr && a.in_stride == N && a.out_stride == N) {
-        if constexpr (std::is_same<TIn, __half2>::value) {
-          if (a.fs_h16) return launch_fourstep_n<N, TIn, MODE, SCALED, true>(a, stream);
-        }
-        return launch_fourstep_n<N, TIn, MODE, SCALED>(a, stream);
+      constexpr bool kHalf = std::is_same<TIn, __half2>::value;
+      if (a.tw_long != nullptr && a.in_stride == N && a.out_stride == N) {
+        const bool h16 = kHalf && a.fs_h16;   // rows handed over as FP16 words
+        if (a.lines * N >= kLongMinPoints)
+          return h16 ? launch_long_n<N, TIn, MODE, SCALED, kHalf>(a, stream)
+                     : launch_long_n<N, TIn, MODE, SCALED>(a, stream);
+        return h16 ? launch_fourstep_n<N, TIn, MODE, SCALED, kHalf>(a, stream)
+                   : launch_fourstep_n<N, TIn, MODE, SCALED>(a, stream);
       }
     }
   }

@@ -159,6 +159,19 @@ __global__ void wide_twiddle_kernel(float2* tw, int ns, int radix, int off) {
   tw[off + 2 * ((q / 2) * ns + k) + (q & 1)] = make_float2(float(c), float(s));
 }
 
+// Column factors of long_rows.cuh for lines of n = a * 1024 points: w = W_n^n2,
+// powers 1 ... 7 and 8, 16, ..., a - 8 as factor f of column n2 at entry
+// 2 ((f / 2) 1024 + n2) + (f & 1).  FP64 sincospi, rounded once to FP32.
+__global__ void long_factor_kernel(float2* tw, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int f = i / 1024, n2 = i % 1024;
+  if (f >= 6 + n / 8192) return;
+  const int e = f < 7 ? f + 1 : 8 * (f - 6);
+  double s, c;
+  sincospi(-2.0 * double((long long)n2 * e) / double(n), &s, &c);
+  tw[2 * ((f / 2) * 1024 + n2) + (f & 1)] = make_float2(float(c), float(s));
+}
+
 // The passes of a line of 2^log2n points: first radix (= points per thread)
 // and the radices after it (0: none).
 struct WidePlan {
@@ -182,7 +195,8 @@ WidePlan wide_plan(int log2n) {
 // Per-device, per-length twiddle tables, created on first use and kept for
 // the life of the process (a few hundred KB per device at most).  Keys
 // 0..16: pass-major Stockham tables; 100 + log2 n: four-step tables;
-// 500 + log2 n: two-pass tables; 600 + log2 n: wide_rows.cuh's tables.
+// 500 + log2 n: two-pass tables; 600 + log2 n: wide_rows.cuh's tables;
+// 700 + log2 n: long_rows.cuh's column factors; 700: its 1024 = 64 x 16 rows.
 std::mutex g_tw_mutex;
 std::map<std::pair<int, int>, float2*> g_tw;
 
@@ -198,16 +212,21 @@ int get_twiddles(int log2n, float2** out) {
     return BFPFFT_OK;
   }
   if (fault("alloc")) return BFPFFT_ERR_OOM;
-  const bool wide = log2n >= 600;
-  const bool two = !wide && log2n >= 500;
-  const bool four = !wide && !two && log2n >= 100;
-  const int n = 1 << (wide ? log2n - 600 : two ? log2n - 500 : four ? log2n - 100 : log2n);
+  const bool lng = log2n >= 700;
+  const bool wide = !lng && log2n >= 600;
+  const bool two = !lng && !wide && log2n >= 500;
+  const bool four = !lng && !wide && !two && log2n >= 100;
+  const int n = 1 << (lng ? (log2n > 700 ? log2n - 700 : 10) : wide ? log2n - 600 : two ? log2n - 500 : four ? log2n - 100 : log2n);
   float2* tw = nullptr;
   const WidePlan wp = wide ? wide_plan(log2n - 600) : WidePlan{0, 0, 0};
   const int second = wp.first * wp.second;   // entries of the second pass (all of them, or the third's offset)
   e = cudaMalloc(&tw, sizeof(float2) * size_t(wide && wp.third ? n + second : n));
   if (e != cudaSuccess) return cuda_status(e);
-  if (wide) {
+  if (log2n == 700) {
+    wide_twiddle_kernel<<<(n + 255) / 256, 256>>>(tw, 64, 16, 0);
+  } else if (lng) {
+    long_factor_kernel<<<(6 + n / 8192) * 4, 256>>>(tw, n);
+  } else if (wide) {
     wide_twiddle_kernel<<<(second + 255) / 256, 256>>>(tw, wp.first, wp.second, 0);
     if (wp.third) wide_twiddle_kernel<<<(n + 255) / 256, 256>>>(tw, second, wp.third, second);
   } else if (two) {
@@ -384,12 +403,13 @@ int get_tc_matrix(void** out) {
 }
 
 // Tables of the kernels that go by the length: wide_rows.cuh's for 512 ..
-// 16384 points; the 4096-point row table and the four-step table of their
-// length for the four-step kernel's 8192 points and more.
+// 16384 points, long_rows.cuh's for 32768 and 65536; the 4096-point row table
+// and the four-step table of their length for the four-step lines' 8192 points
+// and more.
 int length_tables(int log2n, bfp::RowArgs* a) {
   a->tw_line = nullptr;
   a->tw_4step = nullptr;
-  a->tw_wide = nullptr;
+  a->tw_wide = a->tw_long = a->tw_row1024 = nullptr;
   float2* t = nullptr;
   int st = BFPFFT_OK;
   if (log2n >= bfp::kWideMinLog2 && log2n <= bfp::kWideMaxLog2) {
@@ -397,6 +417,12 @@ int length_tables(int log2n, bfp::RowArgs* a) {
     a->tw_wide = reinterpret_cast<const float4*>(t);
   }
   if (log2n < 13) return BFPFFT_OK;
+  if (log2n >= 15) {
+    if ((st = get_twiddles(700 + log2n, &t)) != BFPFFT_OK) return st;
+    a->tw_long = reinterpret_cast<const float4*>(t);
+    if ((st = get_twiddles(700, &t)) != BFPFFT_OK) return st;
+    a->tw_row1024 = reinterpret_cast<const float4*>(t);
+  }
   st = get_twiddles(12, &t);
   if (st != BFPFFT_OK) return st;
   a->tw_line = t;
@@ -453,6 +479,8 @@ struct bfpfft_plan_s {
   int device;
   float2* tw;          // shared tables from the per-device cache (not owned): RowArgs' fields
   const float4* tw_wide = nullptr;
+  const float4* tw_long = nullptr;
+  const float4* tw_row1024 = nullptr;
   const float2* tw_line = nullptr;
   const float2* tw_4step = nullptr;
   int* status;         // the plan's own device status word (owned): timeouts, non-finite outputs
@@ -1005,6 +1033,8 @@ int bfpfft_plan_create(bfpfft_plan* out, int64_t n, int64_t batch, int dtype, in
     return st;
   }
   p->tw_wide = tables.tw_wide;
+  p->tw_long = tables.tw_long;
+  p->tw_row1024 = tables.tw_row1024;
   p->tw_line = tables.tw_line;
   p->tw_4step = tables.tw_4step;
   tune_on_create(p);
@@ -1183,6 +1213,8 @@ int bfpfft_exec(bfpfft_plan plan, const void* in, void* out, void* stream) {
     if (stc != BFPFFT_OK) return stc;
   }
   a.tw_wide = plan->tw_wide;
+  a.tw_long = plan->tw_long;
+  a.tw_row1024 = plan->tw_row1024;
   a.tw_line = plan->tw_line;
   a.tw_4step = plan->tw_4step;
   a.lines = plan->batch;
