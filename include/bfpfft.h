@@ -130,7 +130,9 @@ int bfpfft_plan_destroy(bfpfft_plan plan);
 /*
  * Uneven batch: `count` transforms of lengths n[i] (powers of two in
  * [16, 65536], mixed freely) at point offsets offset_pts[i] of the in / out
- * buffers, by default all computed by ONE persistent launch.  The plan sorts
+ * buffers.  By default batches of fewer than 2^23 points are all computed by
+ * ONE persistent launch, larger ones by one launch per length
+ * (BFPFFT_MANY_PER_LENGTH).  For the persistent launch the plan sorts
  * the lines into tasks of 65,536 points of one length, largest length first;
  * thread-block clusters of 16 CTAs take every clusters-th task in turn (a
  * line of 65536 spans the whole cluster, shorter lines one CTA or part of
@@ -205,8 +207,8 @@ int bfpfft_plan_info(bfpfft_plan plan, int64_t* tasks, int64_t* clusters);
 
 /*
  * bfpfft_exec through a CUDA graph: the first call for a given (in, out) pair
- * captures the plan's launches (for an uneven plan: the task-counter reset
- * and the persistent kernel) into a graph and instantiates it; every call
+ * captures the plan's launches (for an uneven plan: the persistent kernel or
+ * the launch per length) into a graph and instantiates it; every call
  * then launches that graph on `stream`.  A new (in, out) pair re-captures.
  * The graph belongs to the plan and is freed by bfpfft_plan_destroy.
  * Errors: as bfpfft_exec.

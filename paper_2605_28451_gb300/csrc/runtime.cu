@@ -495,8 +495,10 @@ struct bfpfft_plan_s {
   int long_twopass = 0;                 // lines of 32768 / 65536 points by the two-pass kernels (1) or in the
                                         // persistent kernel's four-step lines (0)
   int fs_h16 = 0;                       // FP16 storage: four-step lines exchange their rows as FP16 words (1)
-  int per_length = 0;                   // one dense-row launch per length over its listed lines (1) instead of
-                                        // the persistent kernel
+  int per_length = -1;                  // one dense-row launch per length over its listed lines (1), the persistent
+                                        // kernel (0), or by the batch's size (-1, see large_batch)
+  bool large_batch = false;             // at least kPerLengthPoints points
+  std::mutex fork_mutex;                // the side stream and the two events below serve one exec at a time
   int has_fourstep = 0;                 // some line has 8192 points or more
   long long len_first[kMaxLog2 + 1] = {};   // lines of 2^l points: first index into d_line_off ...
   long long len_count[kMaxLog2 + 1] = {};   // ... and count
@@ -512,7 +514,6 @@ struct bfpfft_plan_s {
   bfp::UnevenTask* d_tasks = nullptr;
   const float2** d_tw = nullptr;
   const float2** d_tw4 = nullptr;
-  int* d_counter = nullptr;
   int num_tasks = 0;
   int clusters = 0;
   // Graph cache of bfpfft_exec_graph.
@@ -524,6 +525,14 @@ struct bfpfft_plan_s {
 
 namespace {
 
+// Uneven batches from this many points on run as one launch per length unless
+// told otherwise: the dense kernels of each length beat the persistent one,
+// whose CTAs are sized for every length at once, as soon as a length fills the
+// GPU (lengths 256 ... 65536, FP16, us per batch, persistent / per length: 2.2 M
+// points 23 / 31, 7.1 M 51 / 43, 25.7 M 166 / 106, 252 M 1545 / 780; lengths
+// 16 ... 1024: 2.8 M 20 / 29, 6.9 M 30 / 34).
+constexpr int64_t kPerLengthPoints = int64_t(1) << 23;
+
 void free_plan_resources(bfpfft_plan p) {
   if (p->graph) cudaGraphExecDestroy(p->graph);
   if (p->status) cudaFree(p->status);
@@ -531,7 +540,6 @@ void free_plan_resources(bfpfft_plan p) {
   if (p->d_tasks) cudaFree(p->d_tasks);
   if (p->d_tw) cudaFree(p->d_tw);
   if (p->d_tw4) cudaFree(p->d_tw4);
-  if (p->d_counter) cudaFree(p->d_counter);
   if (p->side) cudaStreamDestroy(p->side);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
@@ -627,6 +635,7 @@ extern "C" int bfpfft_exec(bfpfft_plan plan, const void* in, void* out, void* st
 // lengths on the plan's side stream forked from it (an event each way, so a
 // stream capture takes both branches), so that their launches overlap.
 static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(plan->fork_mutex);   // host threads may share a plan
   const bool dev_mem = device_memory(in);
   const int mode = plan->direction == BFPFFT_INVERSE ? bfp::kInverse : bfp::kForward;
   bool has_long = false, has_short = false;
@@ -676,7 +685,10 @@ static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStre
 }
 
 static int exec_many(bfpfft_plan plan, const void* in, void* out, cudaStream_t s) {
-  if (plan->per_length) return exec_per_length(plan, in, out, s);
+  // An untuned plan goes by its size, unless BFPFFT_ROWS names a form of the
+  // persistent kernel.
+  const bool by_size = plan->per_length < 0 && plan->large_batch && std::getenv("BFPFFT_ROWS") == nullptr;
+  if (plan->per_length > 0 || by_size) return exec_per_length(plan, in, out, s);
   bfp::UnevenArgs a{};
   a.in = in;
   a.out = out;
@@ -706,7 +718,6 @@ static int exec_many(bfpfft_plan plan, const void* in, void* out, cudaStream_t s
   }
   a.tw = plan->d_tw;
   a.tw4 = plan->d_tw4;
-  a.counter = plan->d_counter;
   a.status = plan->status;
   a.finite_flag = (plan->flags & BFPFFT_CHECK_FINITE) ? plan->status : nullptr;
   // BFPFFT_ROWS naming an FP16-exchange variant forces the FP16 row exchange
@@ -1089,6 +1100,9 @@ int bfpfft_plan_create_many(bfpfft_plan* out, int64_t count, const int64_t* n, c
   p->many = true;
   p->kind = kind;
   p->num_tasks = int(tasks.size());
+  int64_t points = 0;
+  for (int64_t i = 0; i < count; ++i) points += n[i];
+  p->large_batch = points >= kPerLengthPoints;
   // Tasks are sorted longest first: lines of 65536 and 32768 points come first.
   p->first_short_task = 0;
   for (const auto& t : tasks) {
@@ -1128,7 +1142,6 @@ int bfpfft_plan_create_many(bfpfft_plan* out, int64_t count, const int64_t* n, c
     if (e == cudaSuccess) e = cudaMalloc(&p->d_tasks, sizeof(bfp::UnevenTask) * tasks.size());
     if (e == cudaSuccess) e = cudaMalloc(&p->d_tw, sizeof(tw_host));
     if (e == cudaSuccess) e = cudaMalloc(&p->d_tw4, sizeof(tw4_host));
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_counter, sizeof(int));
     if (e == cudaSuccess)
       e = cudaMemcpy(p->d_line_off, line_off.data(), sizeof(long long) * line_off.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)

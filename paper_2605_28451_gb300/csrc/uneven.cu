@@ -264,10 +264,8 @@ cudaError_t uneven_max_clusters(int kind, bool inverse, int* max_clusters) {
 }
 
 cudaError_t launch_uneven(int kind, bool inverse, const UnevenArgs& a, int clusters, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  e = inverse ? dispatch<kInverse>(kind, false, &a, clusters, nullptr, s)
-              : dispatch<kForward>(kind, false, &a, clusters, nullptr, s);
+  const cudaError_t e = inverse ? dispatch<kInverse>(kind, false, &a, clusters, nullptr, s)
+                                : dispatch<kForward>(kind, false, &a, clusters, nullptr, s);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

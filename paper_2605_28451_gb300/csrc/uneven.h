@@ -22,7 +22,6 @@ struct UnevenArgs {
   int num_tasks;
   const float2* const* tw;       // per-length twiddle tables, indexed by log2 N
   const float2* const* tw4;      // per-length four-step tables (N >= 8192), indexed by log2 N
-  int* counter;                  // task counter (reset before every launch)
   int* status;
   int prefetch;                  // nonzero: prefetch each CTA's lines of the next task into L2
   int* finite_flag;              // non-null: record non-finite outputs here (BFPFFT_CHECK_FINITE)
