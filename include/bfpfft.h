@@ -490,8 +490,10 @@ int sar_rda_image(const void* raw, int raw_dtype, void* img, int img_dtype, cons
  *   S = sum q,  E = -sum (q/S) ln(q/S) = ln S - (1/S) sum q ln q,
  *   dE/dphi[n] = 2 sum_r Im( conj((A^H G)[r][n]) v[r][n] ),
  *   G = -(ln(q/S) + E) / S . I,  A^H = IDFT(DFT(.) . conj(Ha)).
- * The image is never stored: the gradient pass recomputes the forward
- * transforms.  FP32 arithmetic; FP64 sums across CTAs.
+ * A gradient call keeps the image (FP32) between its two passes in scratch from
+ * the library's stream-ordered pool, up to 512 MiB; where it does not fit, and
+ * inside a stream capture, the gradient pass computes the forward transforms
+ * again.  FP32 arithmetic; FP64 sums across CTAs.
  * Layout: rc is [n_rg][n_az] (each row one range bin's azimuth line, as written
  * by sar_range_compress with transpose_out = 1), dtype BFPFFT_F32 or
  * BFPFFT_F16_BFP; phi float[n_az], Ha float2[n_az] (device).
@@ -516,8 +518,26 @@ int sar_autofocus_grad(const void* rc, int rc_dtype, const float* phi, const voi
                        void* stream);
 
 /*
- * The same two calls in a chosen arithmetic: BFPFFT_ARITH_F32 is the calls
- * above; BFPFFT_ARITH_F16_MUL_F32_ACC runs every transform on the tensor cores
+ * Entropy and gradient of one point as two calls (an autograd forward and
+ * backward) without computing the image twice: the first leaves its statistics
+ * and the FP32 image in `state`, sar_autofocus_state_bytes() of the caller's
+ * device memory (0 if unsupported); the second takes that state with the same
+ * rc, phi and ha.  entropy_out (device double, may be NULL) receives E; scale
+ * (device double, may be NULL) multiplies the gradient, as FP32.  Same
+ * workspace; FP32 arithmetic.  Errors as above; INVALID_ARG also for a state
+ * that is too small or not device memory.
+ */
+size_t sar_autofocus_state_bytes(int64_t n_az, int64_t n_rg);
+int sar_autofocus_entropy_keep(const void* rc, int rc_dtype, const float* phi, const void* ha, int64_t n_az,
+                               int64_t n_rg, void* stats_out, double* entropy_out, void* state, size_t state_bytes,
+                               void* workspace, size_t ws_bytes, void* stream);
+int sar_autofocus_grad_kept(const void* rc, int rc_dtype, const float* phi, const void* ha, int64_t n_az,
+                            int64_t n_rg, const void* state, size_t state_bytes, const double* scale,
+                            float* grad_out, void* stats_out, void* workspace, size_t ws_bytes, void* stream);
+
+/*
+ * sar_autofocus_entropy and sar_autofocus_grad in a chosen arithmetic:
+ * BFPFFT_ARITH_F32 is those calls; BFPFFT_ARITH_F16_MUL_F32_ACC runs every transform on the tensor cores
  * (FP16 operands at each radix-16 pass, FP32 accumulation; the filter product,
  * |I|^2, the logarithms and all sums in FP32 / FP64 as above), n_az = 4096
  * only.  The gradient pass scales G by a power of two taken from the largest

@@ -1,10 +1,13 @@
 """Differentiable entropy autofocus: a torch.autograd.Function over the C ABI.
 
-Forward calls ``sar_autofocus_entropy`` (image entropy E(phi) of the
-azimuth-compressed, phase-corrected data; the image is never stored).
-Backward calls ``sar_autofocus_grad``, the hand-written adjoint, which
-recomputes the forward transforms on the GPU instead of keeping them.  Only
-argument marshalling happens here.
+Forward computes the image entropy E(phi) of the azimuth-compressed,
+phase-corrected data.  When a gradient will be asked for it also keeps the
+FP32 image (up to KEEP_BYTES) for backward, which then runs the hand-written
+adjoint alone: four transforms per range bin for a step instead of eight.
+Without the image (evaluation only, larger scenes, no memory for it, the
+tensor-core mode, rc or ha changed in place in between) backward calls
+``sar_autofocus_grad``, which computes it again.  Only argument marshalling
+happens here.
 """
 
 from __future__ import annotations
@@ -28,33 +31,55 @@ class Workspace:
         self.stats = torch.empty(4, dtype=torch.float64, device=device)
 
 
+KEEP_BYTES = 512 << 20   # largest state kept between forward and backward
+
+
 class SarEntropy(torch.autograd.Function):
     """E = entropy(|A(rc . exp(-j phi))|^2); d E / d phi by the GPU adjoint.
 
     rc: device tensor [n_rg][n_az] in storage dtype rc_dtype (complex64 for
     BFPFFT_F32, float16 [n_rg][n_az][2] for BFPFFT_F16_BFP); ha: complex64
     [n_az]; phi: float32 [n_az] (requires grad).  Returns a float64 scalar.
+    keep: backward will be asked for, so the image may be kept.
     """
 
     @staticmethod
-    def forward(ctx, phi, rc, ha, rc_dtype: int, ws: Workspace):
+    def forward(ctx, phi, rc, ha, rc_dtype: int, ws: Workspace, keep: bool = False):
         n_rg, n_az = rc.shape[0], rc.shape[1]
         phi_c = phi.detach().contiguous()
+        ctx.rc, ctx.ha, ctx.rc_dtype, ctx.ws = rc, ha, rc_dtype, ws
+        if keep and ws.arith == B.ARITH_F32 and n_rg > 0:
+            size = B.sar_autofocus_state_bytes(n_az, n_rg)
+            if 0 < size <= KEEP_BYTES:
+                try:
+                    state = torch.empty(size, dtype=torch.uint8, device=phi_c.device)
+                except torch.cuda.OutOfMemoryError:
+                    state = None
+                if state is not None:
+                    e = torch.empty((), dtype=torch.float64, device=phi_c.device)
+                    B.sar_autofocus_entropy_keep(rc, rc_dtype, phi_c, ha, n_az, n_rg, ws.stats, e, state, size,
+                                                 ws.buf, ws.bytes)
+                    ctx.save_for_backward(phi_c, state)
+                    ctx.versions = (rc._version, ha._version)
+                    return e
         B.sar_autofocus_entropy(rc, rc_dtype, phi_c, ha, n_az, n_rg, ws.stats, ws.buf, ws.bytes, arith=ws.arith)
         ctx.save_for_backward(phi_c)
-        ctx.rc, ctx.ha, ctx.rc_dtype, ctx.ws = rc, ha, rc_dtype, ws
         return ws.stats[2].clone()
 
     @staticmethod
     def backward(ctx, g_e):
-        (phi_c,) = ctx.saved_tensors
+        phi_c, *kept = ctx.saved_tensors
         rc, ha, ws = ctx.rc, ctx.ha, ctx.ws
         n_rg, n_az = rc.shape[0], rc.shape[1]
         grad = torch.empty(n_az, dtype=torch.float32, device=phi_c.device)
-        B.sar_autofocus_grad(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, grad, ws.stats, ws.buf, ws.bytes,
-                             arith=ws.arith)
-        return (g_e.to(torch.float32) * grad), None, None, None, None
+        if kept and ws.arith == B.ARITH_F32 and ctx.versions == (rc._version, ha._version):
+            state = kept[0]
+            B.sar_autofocus_grad_kept(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, state, state.numel(), g_e, grad,
+                                      ws.stats, ws.buf, ws.bytes)
+            return grad, None, None, None, None, None
+        B.sar_autofocus_grad(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, grad, ws.stats, ws.buf, ws.bytes, arith=ws.arith)
+        return (g_e.to(torch.float32) * grad), None, None, None, None, None
 
 
 def entropy(phi, rc, ha, rc_dtype: int, ws: Workspace):
-    return SarEntropy.apply(phi, rc, ha, rc_dtype, ws)
+    return SarEntropy.apply(phi, rc, ha, rc_dtype, ws, phi.requires_grad and torch.is_grad_enabled())

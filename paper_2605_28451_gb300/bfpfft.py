@@ -95,6 +95,11 @@ SIGNATURES = {
                                                    ctypes.c_size_t, ctypes.c_int, _vp]),
     "sar_autofocus_grad_arith": (ctypes.c_int, [_vp, ctypes.c_int, _vp, _vp, _c_int64, _c_int64, _vp, _vp, _vp,
                                                 ctypes.c_size_t, ctypes.c_int, _vp]),
+    "sar_autofocus_state_bytes": (ctypes.c_size_t, [_c_int64, _c_int64]),
+    "sar_autofocus_entropy_keep": (ctypes.c_int, [_vp, ctypes.c_int, _vp, _vp, _c_int64, _c_int64, _vp, _vp, _vp,
+                                                  ctypes.c_size_t, _vp, ctypes.c_size_t, _vp]),
+    "sar_autofocus_grad_kept": (ctypes.c_int, [_vp, ctypes.c_int, _vp, _vp, _c_int64, _c_int64, _vp, ctypes.c_size_t,
+                                               _vp, _vp, _vp, _vp, ctypes.c_size_t, _vp]),
     "sar_point_target_workspace_bytes": (ctypes.c_size_t, [_c_int64, _c_int64]),
     "sar_point_target_metrics": (ctypes.c_int, [_vp, ctypes.c_int, _c_int64, _c_int64, _vp, _c_int64, ctypes.c_int,
                                                 _vp, _vp, ctypes.c_size_t, _vp]),
@@ -368,6 +373,27 @@ def sar_autofocus_grad(rc, rc_dtype: int, phi, ha, n_az: int, n_rg: int, grad_ou
     _check(lib().sar_autofocus_grad_arith(_ptr(rc), int(rc_dtype), _ptr(phi), _ptr(ha), int(n_az), int(n_rg),
                                           _ptr(grad_out), _ptr(stats_out), _ptr(workspace), int(ws_bytes),
                                           int(arith), _stream(stream)), "sar_autofocus_grad")
+
+
+def sar_autofocus_state_bytes(n_az: int, n_rg: int) -> int:
+    return int(lib().sar_autofocus_state_bytes(int(n_az), int(n_rg)))
+
+
+def sar_autofocus_entropy_keep(rc, rc_dtype: int, phi, ha, n_az: int, n_rg: int, stats_out, entropy_out, state,
+                               state_bytes: int, workspace, ws_bytes: int, stream=None):
+    """Entropy statistics, E, and the state (statistics and image) for sar_autofocus_grad_kept."""
+    _check(lib().sar_autofocus_entropy_keep(_ptr(rc), int(rc_dtype), _ptr(phi), _ptr(ha), int(n_az), int(n_rg),
+                                            _ptr(stats_out), _ptr(entropy_out), _ptr(state), int(state_bytes),
+                                            _ptr(workspace), int(ws_bytes), _stream(stream)),
+           "sar_autofocus_entropy_keep")
+
+
+def sar_autofocus_grad_kept(rc, rc_dtype: int, phi, ha, n_az: int, n_rg: int, state, state_bytes: int, scale,
+                            grad_out, stats_out, workspace, ws_bytes: int, stream=None):
+    _check(lib().sar_autofocus_grad_kept(_ptr(rc), int(rc_dtype), _ptr(phi), _ptr(ha), int(n_az), int(n_rg),
+                                         _ptr(state), int(state_bytes), _ptr(scale), _ptr(grad_out),
+                                         _ptr(stats_out), _ptr(workspace), int(ws_bytes), _stream(stream)),
+           "sar_autofocus_grad_kept")
 
 
 def bfp_sqnr_sums_noalloc_max_count() -> int:

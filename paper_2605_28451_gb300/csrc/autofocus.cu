@@ -14,11 +14,19 @@
 //
 // Kernels (persistent, one group of N/16 threads per range bin, lines held on
 // chip exactly as in fft_rows.cuh):
-//   af_phase_kernel     e^{-j phi[n]} table
-//   af_kernel<fwd>      per-CTA FP64 partials of S and sum q ln q
-//   af_stats_kernel     S, Q, E, ln S (one block, FP64 tree over the partials)
-//   af_kernel<bwd>      per-CTA partial gradients (registers across rows)
-//   af_grad_kernel      sum of the partial gradients in FP64 (8 slices per 32 pulses)
+//   af_phase_kernel         e^{-j phi[n]} table
+//   af_kernel<kAfEntropy>   per-CTA FP64 partials of S and sum q ln q; for a gradient
+//                           it also keeps I[r] (FP32) in scratch, where there is room
+//   af_stats_kernel         S, Q, E, ln S (one block, FP64 tree over the partials)
+//   af_kernel<kAfAdjoint>   per-CTA partial gradients from the kept I
+//   af_kernel<kAfRecompute> the same without scratch: I[r] is computed again
+//   af_grad_kernel          sum of the partial gradients in FP64 (32 slices per 32 pulses)
+//
+// Arithmetic bounds the passes (FMA pipe 50 to 60 % busy), so a gradient step
+// costs its transforms: four with I kept, six when it is computed again.  Kept,
+// I moves 16 bytes a pixel more through L2 and HBM, which the arithmetic
+// covers.  Measured on GB300, 4096 x 4096 FP16 rc, one gradient step: see
+// kAfKeepBytes.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -33,6 +41,7 @@ namespace {
 
 struct AfArgs {
   const void* rc;
+  float2* img;           // I [n_rg][n_az]: written by the entropy pass when not null, read by kAfAdjoint
   const float2* ph;      // e^{-j phi[n]}
   const float2* ha;
   const float2* tw;
@@ -54,15 +63,17 @@ __global__ void af_phase_kernel(const float* __restrict__ phi, float2* __restric
 
 // One compression of the line held in v with filter h (conjugated if CONJ_H):
 // v <- conj(DFT(conj(DFT(v) . h) / N)).
-template <int N, bool CONJ_H>
+template <int N, bool CONJ_H, bool OPAQUE = false>
 __device__ __forceinline__ void af_compress(float2 (&v)[kPointsPerThread], const float2* __restrict__ h,
                                             const float2* __restrict__ tw, float2* sm, int t) {
   constexpr int P = kPointsPerThread, T = N / P;
   const float inv_n = 1.0f / float(N);
-  // Fresh opaque copies of t for each transform: the compiler must not keep
-  // one transform's shared-memory and twiddle addresses live for the next.
-  int t1;
-  asm volatile("mov.b32 %0, %1;" : "=r"(t1) : "r"(t));
+  // The second transform runs on an opaque copy of t: the compiler must not
+  // keep the first one's shared-memory and twiddle addresses live for it.  With
+  // OPAQUE (four transforms in one kernel) so does the first; in the kernels
+  // of two transforms that spills 250 to 580 bytes at 64 registers.
+  int t1 = t;
+  if (OPAQUE) asm volatile("mov.b32 %0, %1;" : "=r"(t1) : "r"(t));
   line_dft<N>(v, tw, sm, t1);
   // Filter loads in groups of four, so the compiler does not hoist all
   // sixteen next to the line (register pressure at 3 CTAs / SM).
@@ -112,31 +123,39 @@ __device__ __forceinline__ void af_load(float2 (&v)[kPointsPerThread], const AfA
   }
 }
 
-// Shared memory of af_kernel: the row buffers, and for the gradient pass one
-// FP32 partial gradient per pulse for each line group of the CTA (a thread
-// owns the pulses t + T m of its group's slice, so no atomics are needed).
-template <int N, bool BACKWARD>
-constexpr size_t af_smem_bytes() {
-  using S = RowShape<N>;
-  return S::kSmemBytes + (BACKWARD ? size_t(S::G) * N * sizeof(float) : 0);
+enum AfPass : int { kAfEntropy = 0, kAfAdjoint = 1, kAfRecompute = 2 };
+
+// Resident CTAs per SM: 64 registers (4 CTAs of 256 threads, 2 of 512) for the
+// entropy pass, as the compression lines; 128 for the gradient passes, whose
+// threads also keep the partial gradients of their pulses (more CTAs spill and
+// leave more partials to sum: 4 per SM 249 us a step, 2 per SM 224).
+template <int N, int PASS>
+constexpr int af_min_blocks() {
+  return PASS == kAfEntropy ? RowShape<N>::kMinBlocksDense : RowShape<N>::kThreads >= 512 ? 1 : 2;
 }
 
-template <int N, class TIn, bool BACKWARD>
-__global__ void __launch_bounds__(RowShape<N>::kThreads, RowShape<N>::kThreads >= 512 ? 1 : 2)
+template <int N, class TIn, int PASS>
+__global__ void __launch_bounds__(RowShape<N>::kThreads, af_min_blocks<N, PASS>())
 af_kernel(const AfArgs a) {
   using S = RowShape<N>;
   constexpr int P = S::P, T = S::T, G = S::G;
+  constexpr bool BACKWARD = PASS != kAfEntropy;
   extern __shared__ float2 smem_af[];
   const int g = threadIdx.x / T;
   const int t = threadIdx.x - g * T;
   float2* sm = smem_af + g * S::kSmemPerLine;
-  float* gsm = reinterpret_cast<float*>(smem_af + G * S::kSmemPerLine) + g * N;   // this group's gradients
   const long long groups = (a.rows + G - 1) / G;
 
   float s_acc = 0.f, q_acc = 0.f;
-  if (BACKWARD) {
+  // Gradient passes: the sums of this thread's pulses t + T m over the group's
+  // rows, in registers; kAfRecompute, short of those, keeps them in shared memory.
+  constexpr bool kShared = PASS == kAfRecompute;
+  float* gsm = reinterpret_cast<float*>(smem_af + (kShared ? G * S::kSmemPerLine : 0)) + g * N;
+  float grad[P];
 #pragma unroll
-    for (int m = 0; m < P; ++m) gsm[t + T * m] = 0.f;
+  for (int m = 0; m < P; ++m) {
+    grad[m] = 0.f;
+    if (kShared) gsm[t + T * m] = 0.f;
   }
   float ln_s_minus_e = 0.f, inv_s = 0.f;
   if (BACKWARD) {
@@ -144,20 +163,30 @@ af_kernel(const AfArgs a) {
     inv_s = float(1.0 / a.stats[0]);
   }
 
-  for (long long grp = blockIdx.x; grp < groups; grp += gridDim.x) {
-    if (a.prefetch && threadIdx.x == 0 && grp + gridDim.x < groups) {
+  for (long long i = blockIdx.x; i < groups; i += gridDim.x) {
+    // The adjoint pass takes the rows last written first: those are in L2.
+    const long long grp = PASS == kAfAdjoint ? groups - 1 - i : i;
+    if (i + gridDim.x < groups && threadIdx.x == 0) {
       // The rows of this CTA's next group, into L2.
-      const long long r0 = (grp + gridDim.x) * G;
+      const long long r0 = (PASS == kAfAdjoint ? grp - gridDim.x : grp + gridDim.x) * G;
       const long long cnt = a.rows - r0 < G ? a.rows - r0 : G;
-      prefetch_l2_bulk(static_cast<const TIn*>(a.rc) + r0 * N, uint32_t(cnt * N * sizeof(TIn)));
+      if (a.prefetch)
+        prefetch_l2_bulk(static_cast<const TIn*>(a.rc) + r0 * N, uint32_t(cnt * N * sizeof(TIn)));
+      if (PASS == kAfAdjoint) prefetch_l2_bulk(a.img + r0 * N, uint32_t(cnt * N * sizeof(float2)));
     }
     const long long row = grp * G + g;
     const bool active = row < a.rows;
-    int ti;
-    asm volatile("mov.b32 %0, %1;" : "=r"(ti) : "r"(t));
+    int ti = t;
+    if (PASS == kAfRecompute) asm volatile("mov.b32 %0, %1;" : "=r"(ti) : "r"(t));
     float2 v[P];
-    af_load<N, TIn>(v, a, row, ti, active);
-    af_compress<N, false>(v, a.ha, a.tw, sm, ti);          // v = I[row]
+    if constexpr (PASS == kAfAdjoint) {
+      const float2* img = a.img + row * N + ti;
+#pragma unroll
+      for (int m = 0; m < P; ++m) v[m] = active ? Storage<float2>::load(img + T * m) : make_float2(0.f, 0.f);
+    } else {
+      af_load<N, TIn>(v, a, row, ti, active);
+      af_compress<N, false, PASS == kAfRecompute>(v, a.ha, a.tw, sm, ti);          // v = I[row]
+    }
     if (!BACKWARD) {
       if (active) {
 #pragma unroll
@@ -165,6 +194,11 @@ af_kernel(const AfArgs a) {
           const float q = v[m].x * v[m].x + v[m].y * v[m].y;
           s_acc += q;
           if (q > 0.f) q_acc += q * logf(q);
+        }
+        if (a.img != nullptr) {
+          float2* img = a.img + row * N + ti;
+#pragma unroll
+          for (int m = 0; m < P; ++m) img[T * m] = v[m];
         }
       }
     } else {
@@ -175,7 +209,7 @@ af_kernel(const AfArgs a) {
         const float w = q > 0.f ? (ln_s_minus_e - logf(q)) * inv_s : 0.f;
         v[m] = cscale(v[m], w);
       }
-      af_compress<N, true>(v, a.ha, a.tw, sm, ti);         // v = (A^H G)[row]
+      af_compress<N, true, PASS == kAfRecompute>(v, a.ha, a.tw, sm, ti);         // v = (A^H G)[row]
       if (active) {
         // v[row] again (from L2), four points at a time to bound live registers.
         const TIn* in = static_cast<const TIn*>(a.rc) + row * N + ti;
@@ -183,11 +217,13 @@ af_kernel(const AfArgs a) {
         for (int m0 = 0; m0 < P; m0 += 4) {
           float2 x[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) x[i] = cmul(load_cached(in + T * (m0 + i)), __ldg(a.ph + ti + T * (m0 + i)));
+          for (int j = 0; j < 4; ++j) x[j] = cmul(load_cached(in + T * (m0 + j)), __ldg(a.ph + ti + T * (m0 + j)));
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float2 b = v[m0 + i];
-            gsm[ti + T * (m0 + i)] += 2.f * (b.x * x[i].y - b.y * x[i].x);      // 2 Im(conj(b) x)
+          for (int j = 0; j < 4; ++j) {
+            const float2 b = v[m0 + j];
+            const float d = 2.f * (b.x * x[j].y - b.y * x[j].x);      // 2 Im(conj(b) x)
+            if (kShared) gsm[ti + T * (m0 + j)] += d;
+            else grad[m0 + j] += d;
           }
           asm volatile("" ::: "memory");
         }
@@ -218,15 +254,26 @@ af_kernel(const AfArgs a) {
       a.sq_part[2 * blockIdx.x + 1] = qq;
     }
   } else {
-    // Groups of one CTA cover the same pulses: add their slices.
-    __syncthreads();
-    const float* g0 = reinterpret_cast<const float*>(smem_af + G * S::kSmemPerLine);
+    // Groups of one CTA cover the same pulses: add their sums, by way of the
+    // row buffers (free once every group is past its last exchange).
     float* dst = a.g_part + (long long)blockIdx.x * N;
-    for (int i = threadIdx.x; i < N; i += S::kThreads) {
-      float acc = 0.f;
+    if constexpr (G == 1 && !kShared) {
 #pragma unroll
-      for (int gg = 0; gg < G; ++gg) acc += g0[gg * N + i];
-      dst[i] = acc;
+      for (int m = 0; m < P; ++m) dst[t + T * m] = grad[m];
+    } else {
+      __syncthreads();
+      if (!kShared) {
+#pragma unroll
+        for (int m = 0; m < P; ++m) gsm[t + T * m] = grad[m];
+        __syncthreads();
+      }
+      const float* g0 = gsm - g * N;
+      for (int i = threadIdx.x; i < N; i += S::kThreads) {
+        float acc = 0.f;
+#pragma unroll
+        for (int gg = 0; gg < G; ++gg) acc += g0[gg * N + i];
+        dst[i] = acc;
+      }
     }
   }
 }
@@ -237,7 +284,9 @@ af_kernel(const AfArgs a) {
 constexpr int kAfRedThreads = 256;
 
 __global__ void __launch_bounds__(kAfRedThreads) af_stats_kernel(const double* __restrict__ sq_part, int grid,
-                                                                 double* __restrict__ stats) {
+                                                                 double* __restrict__ stats,
+                                                                 double* __restrict__ kept,
+                                                                 double* __restrict__ entropy) {
   __shared__ double red[2][kAfRedThreads / 32];
   double s = 0.0, q = 0.0;
   for (int b = threadIdx.x; b < grid; b += kAfRedThreads) {
@@ -261,20 +310,31 @@ __global__ void __launch_bounds__(kAfRedThreads) af_stats_kernel(const double* _
       s += red[0][w];
       q += red[1][w];
     }
-    stats[0] = s;
-    stats[1] = q;
-    stats[2] = s > 0.0 ? log(s) - q / s : 0.0;
-    stats[3] = s > 0.0 ? log(s) : 0.0;
+    const double ln_s = s > 0.0 ? log(s) : 0.0;
+    const double e = s > 0.0 ? ln_s - q / s : 0.0;
+    const double out[4] = {s, q, e, ln_s};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      stats[i] = out[i];
+      if (kept != nullptr) kept[i] = out[i];
+    }
+    if (entropy != nullptr) *entropy = e;
   }
 }
 
 // grad[i] = sum over CTAs b of g_part[b][i], in FP64: a block covers 32
-// consecutive pulses (one per lane: coalesced rows) with 8 warps splitting
-// the CTAs between them, then adds the 8 partial sums.
-constexpr int kAfGradSlices = 8;
+// consecutive pulses (one per lane: coalesced rows) with 32 warps splitting
+// the CTAs between them, then adds the 32 partial sums.
+constexpr int kAfGradSlices = 32;
 
+// scale (may be null) multiplies the result, as FP32; `kept` statistics go to
+// stats_out as well.
 __global__ void __launch_bounds__(32 * kAfGradSlices) af_grad_kernel(const float* __restrict__ g_part, int grid,
-                                                                    int n, float* __restrict__ grad) {
+                                                                    int n, float* __restrict__ grad,
+                                                                    const double* __restrict__ scale,
+                                                                    const double* __restrict__ kept,
+                                                                    double* __restrict__ stats_out) {
+  if (stats_out != nullptr && blockIdx.x == 0 && threadIdx.x < 4) stats_out[threadIdx.x] = kept[threadIdx.x];
   __shared__ double red[kAfGradSlices][32];
   const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;
@@ -287,15 +347,15 @@ __global__ void __launch_bounds__(32 * kAfGradSlices) af_grad_kernel(const float
     double t = 0.0;
 #pragma unroll
     for (int k = 0; k < kAfGradSlices; ++k) t += red[k][lane];
-    grad[i] = float(t);
+    grad[i] = scale != nullptr ? float(*scale) * float(t) : float(t);
   }
 }
 
-template <int N, class TIn, bool BACKWARD>
+template <int N, class TIn, int PASS>
 cudaError_t launch_af_n(const AfArgs& a, int* grid_out, cudaStream_t s) {
   using S = RowShape<N>;
-  auto kern = af_kernel<N, TIn, BACKWARD>;
-  constexpr size_t kBytes = af_smem_bytes<N, BACKWARD>();
+  auto kern = af_kernel<N, TIn, PASS>;
+  constexpr size_t kBytes = S::kSmemBytes + (PASS == kAfRecompute ? size_t(S::G) * N * sizeof(float) : 0);
   // One-time, thread-safe set-up (function-local static): resident CTAs,
   // capped by the workspace's partial-gradient slots.
   static const LaunchSetup setup = setup_kernel(kern, S::kThreads, kBytes);
@@ -308,17 +368,22 @@ cudaError_t launch_af_n(const AfArgs& a, int* grid_out, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <class TIn, bool BACKWARD>
-cudaError_t launch_af(int log2n, const AfArgs& a, int* grid, cudaStream_t s) {
+template <class TIn, int PASS>
+cudaError_t launch_af_typed(int log2n, const AfArgs& a, int* grid, cudaStream_t s) {
   switch (log2n) {
-    case 8: return launch_af_n<256, TIn, BACKWARD>(a, grid, s);
-    case 9: return launch_af_n<512, TIn, BACKWARD>(a, grid, s);
-    case 10: return launch_af_n<1024, TIn, BACKWARD>(a, grid, s);
-    case 11: return launch_af_n<2048, TIn, BACKWARD>(a, grid, s);
-    case 12: return launch_af_n<4096, TIn, BACKWARD>(a, grid, s);
-    case 13: return launch_af_n<8192, TIn, BACKWARD>(a, grid, s);
+    case 8: return launch_af_n<256, TIn, PASS>(a, grid, s);
+    case 9: return launch_af_n<512, TIn, PASS>(a, grid, s);
+    case 10: return launch_af_n<1024, TIn, PASS>(a, grid, s);
+    case 11: return launch_af_n<2048, TIn, PASS>(a, grid, s);
+    case 12: return launch_af_n<4096, TIn, PASS>(a, grid, s);
+    case 13: return launch_af_n<8192, TIn, PASS>(a, grid, s);
     default: return cudaErrorInvalidValue;
   }
+}
+
+template <int PASS>
+cudaError_t launch_af(int log2n, bool rc16, const AfArgs& a, int* grid, cudaStream_t s) {
+  return rc16 ? launch_af_typed<__half2, PASS>(log2n, a, grid, s) : launch_af_typed<float2, PASS>(log2n, a, grid, s);
 }
 
 }  // namespace
@@ -348,42 +413,77 @@ cudaError_t af_phase_table(const float* phi, float2* ph, long long n_az, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t af_entropy_stats(const double* sq_part, int grid, double* stats, cudaStream_t s) {
-  af_stats_kernel<<<1, kAfRedThreads, 0, s>>>(sq_part, grid, stats);
+cudaError_t af_entropy_stats(const double* sq_part, int grid, double* stats, cudaStream_t s, double* kept,
+                             double* entropy) {
+  af_stats_kernel<<<1, kAfRedThreads, 0, s>>>(sq_part, grid, stats, kept, entropy);
   return cudaGetLastError();
 }
 
-cudaError_t af_gradient_sum(const float* g_part, int grid, int n_az, float* grad, cudaStream_t s) {
-  af_grad_kernel<<<(n_az + 31) / 32, 32 * kAfGradSlices, 0, s>>>(g_part, grid, n_az, grad);
+cudaError_t af_gradient_sum(const float* g_part, int grid, int n_az, float* grad, cudaStream_t s,
+                            const double* scale, const double* kept, double* stats_out) {
+  af_grad_kernel<<<(n_az + 31) / 32, 32 * kAfGradSlices, 0, s>>>(g_part, grid, n_az, grad, scale, kept, stats_out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_autofocus(int log2n, bool rc16, const void* rc, const float* phi, const float2* ha,
-                             const float2* tw, long long n_rg, double* stats, float* grad, void* workspace,
-                             bool prefetch, cudaStream_t s) {
-  const long long n_az = 1LL << log2n;
-  const AfWorkspaceLayout l = af_workspace_layout(workspace, n_az);
+namespace {
+
+// The kept state: the four statistics, then the image.
+struct AfState {
+  double* stats;
+  float2* image;
+};
+AfState af_state(void* state) {
+  if (state == nullptr) return {nullptr, nullptr};
+  unsigned char* p = static_cast<unsigned char*>(state);
+  return {reinterpret_cast<double*>(p), reinterpret_cast<float2*>(p + kAfStateHead)};
+}
+
+AfArgs af_args(int log2n, const void* rc, const float2* ha, const float2* tw, long long n_rg, double* stats,
+               void* workspace, float2* image, bool prefetch) {
+  const AfWorkspaceLayout l = af_workspace_layout(workspace, 1LL << log2n);
   AfArgs a;
-  a.sq_part = l.sq_part;
-  a.g_part = l.g_part;
-  float2* ph = l.ph;
   a.rc = rc;
-  a.ph = ph;
+  a.img = image;
+  a.ph = l.ph;
   a.ha = ha;
   a.tw = tw;
   a.rows = n_rg;
   a.stats = stats;
+  a.sq_part = l.sq_part;
+  a.g_part = l.g_part;
   a.prefetch = prefetch;
-  cudaError_t e = af_phase_table(phi, ph, n_az, s);
+  return a;
+}
+
+}  // namespace
+
+cudaError_t launch_autofocus_entropy(int log2n, bool rc16, const void* rc, const float* phi, const float2* ha,
+                                     const float2* tw, long long n_rg, double* stats, void* workspace,
+                                     void* state, double* entropy, bool prefetch, cudaStream_t s) {
+  const AfState keep = af_state(state);
+  const AfArgs a = af_args(log2n, rc, ha, tw, n_rg, stats, workspace, keep.image, prefetch);
+  cudaError_t e = af_phase_table(phi, af_workspace_layout(workspace, 1LL << log2n).ph, 1LL << log2n, s);
   if (e != cudaSuccess) return e;
   int grid = 0;
-  e = rc16 ? launch_af<__half2, false>(log2n, a, &grid, s) : launch_af<float2, false>(log2n, a, &grid, s);
+  if ((e = launch_af<kAfEntropy>(log2n, rc16, a, &grid, s)) != cudaSuccess) return e;
+  return af_entropy_stats(a.sq_part, grid, stats, s, keep.stats, entropy);
+}
+
+cudaError_t launch_autofocus_gradient(int log2n, bool rc16, const void* rc, const float* phi, const float2* ha,
+                                      const float2* tw, long long n_rg, double* stats, float* grad, void* workspace,
+                                      void* state, const double* scale, bool prefetch, cudaStream_t s) {
+  const AfState kept = af_state(state);
+  const AfArgs a = af_args(log2n, rc, ha, tw, n_rg, state != nullptr ? kept.stats : stats, workspace, kept.image,
+                           prefetch);
+  cudaError_t e = cudaSuccess;
+  if (phi != nullptr)
+    e = af_phase_table(phi, af_workspace_layout(workspace, 1LL << log2n).ph, 1LL << log2n, s);
   if (e != cudaSuccess) return e;
-  if ((e = af_entropy_stats(a.sq_part, grid, stats, s)) != cudaSuccess) return e;
-  if (grad == nullptr) return cudaSuccess;
-  e = rc16 ? launch_af<__half2, true>(log2n, a, &grid, s) : launch_af<float2, true>(log2n, a, &grid, s);
+  int grid = 0;
+  e = state != nullptr ? launch_af<kAfAdjoint>(log2n, rc16, a, &grid, s)
+                       : launch_af<kAfRecompute>(log2n, rc16, a, &grid, s);
   if (e != cudaSuccess) return e;
-  return af_gradient_sum(a.g_part, grid, int(n_az), grad, s);
+  return af_gradient_sum(a.g_part, grid, 1 << log2n, grad, s, scale, kept.stats, state != nullptr ? stats : nullptr);
 }
 
 }  // namespace bfp

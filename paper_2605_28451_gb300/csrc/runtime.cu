@@ -1750,6 +1750,26 @@ size_t sar_autofocus_workspace_bytes(int64_t n_az) {
   return bfp::af_workspace_bytes(n_az);
 }
 
+// A gradient keeps the FP32 image of its entropy pass in stream-ordered scratch
+// up to this size (16383 range bins of 4096 pulses); beyond it, without memory
+// for it, or inside a stream capture, the gradient pass computes it again.
+// Kept, a gradient step on 4096 x 4096 FP16 data takes 223 us, computed again
+// 289.
+constexpr size_t kAfKeepBytes = size_t(512) << 20;
+
+static void* autofocus_scratch_state(int64_t n_az, int64_t n_rg, cudaStream_t s) {
+  const size_t bytes = bfp::af_state_bytes(n_az, n_rg);
+  if (n_rg == 0 || bytes > kAfKeepBytes) return nullptr;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  void* p = nullptr;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
+      scratch_alloc(&p, bytes, s) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  return p;
+}
+
 static int autofocus_common(const void* rc, int rc_dtype, const float* phi, const void* ha, int64_t n_az,
                             int64_t n_rg, float* grad_out, void* stats_out, void* workspace, size_t ws_bytes,
                             int arith, void* stream) {
@@ -1780,10 +1800,71 @@ static int autofocus_common(const void* rc, int rc_dtype, const float* phi, cons
                                  static_cast<double*>(stats_out), grad_out, tw, device_memory(rc), s);
     return cuda_status(e);
   }
-  cudaError_t e = bfp::launch_autofocus(l, rc_dtype == BFPFFT_F16_BFP, rc, phi, static_cast<const float2*>(ha),
-                                        a.tw, n_rg, static_cast<double*>(stats_out), grad_out, workspace,
-                                        device_memory(rc), s);
-  return cuda_status(e);
+  const bool rc16 = rc_dtype == BFPFFT_F16_BFP, prefetch = device_memory(rc);
+  const float2* h = static_cast<const float2*>(ha);
+  double* stats = static_cast<double*>(stats_out);
+  void* state = grad_out != nullptr ? autofocus_scratch_state(n_az, n_rg, s) : nullptr;
+  cudaError_t e = bfp::launch_autofocus_entropy(l, rc16, rc, phi, h, a.tw, n_rg, stats, workspace, state, nullptr,
+                                                prefetch, s);
+  if (e == cudaSuccess && grad_out != nullptr)
+    e = bfp::launch_autofocus_gradient(l, rc16, rc, nullptr, h, a.tw, n_rg, stats, grad_out, workspace, state,
+                                       nullptr, prefetch, s);
+  const cudaError_t f = state != nullptr ? cudaFreeAsync(state, s) : cudaSuccess;
+  return cuda_status(e != cudaSuccess ? e : f);
+}
+
+size_t sar_autofocus_state_bytes(int64_t n_az, int64_t n_rg) {
+  const int l = log2_exact(n_az);
+  if (l < bfp::kAfMinLog2 || l > bfp::kAfMaxLog2 || n_rg < 0) return 0;
+  return bfp::af_state_bytes(n_az, n_rg);
+}
+
+// Argument checks and set-up shared by the two calls below.
+static int autofocus_kept_check(const void* rc, int rc_dtype, const float* phi, const void* ha, int64_t n_az,
+                                int64_t n_rg, const void* stats, const void* state, size_t state_bytes,
+                                const void* workspace, size_t ws_bytes, bfp::RowArgs* a) {
+  if (n_rg < 0) return BFPFFT_ERR_INVALID_ARG;
+  const int l = log2_exact(n_az);
+  if (l < bfp::kAfMinLog2 || l > bfp::kAfMaxLog2) return BFPFFT_ERR_UNSUPPORTED;
+  if (rc_dtype != BFPFFT_F32 && rc_dtype != BFPFFT_F16_BFP) return BFPFFT_ERR_UNSUPPORTED;
+  if (rc == nullptr || phi == nullptr || ha == nullptr || stats == nullptr || state == nullptr || workspace == nullptr)
+    return BFPFFT_ERR_INVALID_ARG;
+  if (!aligned16(rc) || !aligned16(ha) || !aligned16(stats) || !aligned16(state) || !aligned16(workspace))
+    return BFPFFT_ERR_MISALIGNED;
+  if (ws_bytes < bfp::af_workspace_bytes(n_az) || state_bytes < bfp::af_state_bytes(n_az, n_rg))
+    return BFPFFT_ERR_INVALID_ARG;
+  if (fault("launch")) return BFPFFT_ERR_CUDA;
+  if (!device_memory(state)) return BFPFFT_ERR_INVALID_ARG;
+  return row_args(l, a);
+}
+
+int sar_autofocus_entropy_keep(const void* rc, int rc_dtype, const float* phi, const void* ha, int64_t n_az,
+                               int64_t n_rg, void* stats_out, double* entropy_out, void* state, size_t state_bytes,
+                               void* workspace, size_t ws_bytes, void* stream) {
+  bfp::RowArgs a;
+  const int st = autofocus_kept_check(rc, rc_dtype, phi, ha, n_az, n_rg, stats_out, state, state_bytes, workspace,
+                                      ws_bytes, &a);
+  if (st != BFPFFT_OK) return st;
+  return cuda_status(bfp::launch_autofocus_entropy(log2_exact(n_az), rc_dtype == BFPFFT_F16_BFP, rc, phi,
+                                                   static_cast<const float2*>(ha), a.tw, n_rg,
+                                                   static_cast<double*>(stats_out), workspace, state, entropy_out,
+                                                   device_memory(rc), static_cast<cudaStream_t>(stream)));
+}
+
+int sar_autofocus_grad_kept(const void* rc, int rc_dtype, const float* phi, const void* ha, int64_t n_az,
+                            int64_t n_rg, const void* state, size_t state_bytes, const double* scale,
+                            float* grad_out, void* stats_out, void* workspace, size_t ws_bytes, void* stream) {
+  if (grad_out == nullptr) return BFPFFT_ERR_INVALID_ARG;
+  bfp::RowArgs a;
+  const int st = autofocus_kept_check(rc, rc_dtype, phi, ha, n_az, n_rg, stats_out, state, state_bytes, workspace,
+                                      ws_bytes, &a);
+  if (st != BFPFFT_OK) return st;
+  if (!aligned16(grad_out)) return BFPFFT_ERR_MISALIGNED;
+  return cuda_status(bfp::launch_autofocus_gradient(log2_exact(n_az), rc_dtype == BFPFFT_F16_BFP, rc, phi,
+                                                    static_cast<const float2*>(ha), a.tw, n_rg,
+                                                    static_cast<double*>(stats_out), grad_out, workspace,
+                                                    const_cast<void*>(state), scale, device_memory(rc),
+                                                    static_cast<cudaStream_t>(stream)));
 }
 
 int sar_autofocus_entropy_arith(const void* rc, int rc_dtype, const float* phi, const void* ha, int64_t n_az,
