@@ -18,15 +18,19 @@ struct RdaArgs {
   void* out;               // [lines][N]; may equal in
   const float2* tw;        // pass-major FP32 twiddles of length N
   long long lines;
-  long long other;         // the other dimension: n_az for RCMC lines, n_rg for azimuth lines
-  RdaGeometry geo;
+  const unsigned long long* line_turns;   // per line: its phase unit as a binary fraction of a turn (launch_rda_lines)
   int aperture;            // azimuth chirp length L (pulses)
-  int range_dependent;     // azimuth lines: k_a(R) of the line's own range (else of the centre range)
   int peak_normalise;      // azimuth lines: H_r / max |H_r|
 };
 
 constexpr int kRdaMinLog2 = 8;
 constexpr int kRdaMaxLog2 = 13;
+
+// The phase units of the lines: shift[n_az] for RCMC lines, rate[n_rg] for
+// azimuth lines (range_dependent: k_a of each bin's own range, else of the
+// centre range).
+cudaError_t launch_rda_lines(const RdaGeometry& geo, bool range_dependent, int n_az, int n_rg,
+                             unsigned long long* shift, unsigned long long* rate, cudaStream_t s);
 
 // RCMC lines (along range, one per Doppler bin) and azimuth lines (along
 // Doppler, one per range bin); f16 selects half2 storage, else float2.

@@ -1683,8 +1683,12 @@ int sar_rda_image(const void* raw, int raw_dtype, void* img, int img_dtype, cons
   if (st != BFPFFT_OK) return st;
   void* sa = nullptr;
   void* sb = nullptr;
-  cudaError_t e = scratch_alloc(&sa, bytes, s);
+  cudaError_t e = scratch_alloc(&sa, bytes + size_t(n_az + n_rg) * sizeof(unsigned long long), s);
   if (e == cudaSuccess) e = scratch_alloc(&sb, bytes, s);
+  // 0. the lines' phase units, behind the first scratch array
+  unsigned long long* turns = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(sa) + bytes);
+  if (e == cudaSuccess)
+    e = bfp::launch_rda_lines(geo, (flags & SAR_RDA_RANGE_DEPENDENT) != 0, int(n_az), int(n_rg), turns, turns + n_az, s);
   // 1. range compression: rows of raw into sb [n_az][n_rg], turned into sa [n_rg][n_az]
   if (e == cudaSuccess) {
     ra.in = raw;
@@ -1711,9 +1715,7 @@ int sar_rda_image(const void* raw, int raw_dtype, void* img, int img_dtype, cons
       e = f16 ? bfp::launch_rows_f16(la, bfp::kForward, false, az, s) : bfp::launch_rows_f32(la, bfp::kForward, az, s);
   }
   bfp::RdaArgs r{};
-  r.geo = geo;
   r.aperture = int(aperture);
-  r.range_dependent = (flags & SAR_RDA_RANGE_DEPENDENT) ? 1 : 0;
   r.peak_normalise = (flags & SAR_RDA_PEAK_NORMALISE) ? 1 : 0;
   // 3. RCMC along range, one line per Doppler bin ([f][r] layout)
   if (e == cudaSuccess && (flags & SAR_RDA_RCMC)) {
@@ -1722,7 +1724,7 @@ int sar_rda_image(const void* raw, int raw_dtype, void* img, int img_dtype, cons
     r.out = sb;
     r.tw = ra.tw;
     r.lines = n_az;
-    r.other = n_az;
+    r.line_turns = turns;
     if (e == cudaSuccess) e = bfp::launch_rcmc_rows(lr, f16, r, s);
     if (e == cudaSuccess) e = bfp::launch_transpose(sb, sa, n_az, n_rg, eb, s);
   }
@@ -1732,7 +1734,7 @@ int sar_rda_image(const void* raw, int raw_dtype, void* img, int img_dtype, cons
     r.out = sb;
     r.tw = tw_az;
     r.lines = n_rg;
-    r.other = n_rg;
+    r.line_turns = turns + n_az;
     e = bfp::launch_azimuth_rows(la, f16, r, s);
   }
   // 5. turned into the image [n_az][n_rg]
