@@ -70,8 +70,7 @@ __device__ __forceinline__ void af_compress(float2 (&v)[kPointsPerThread], const
   const float inv_n = 1.0f / float(N);
   // The second transform runs on an opaque copy of t: the compiler must not
   // keep the first one's shared-memory and twiddle addresses live for it.  With
-  // OPAQUE (four transforms in one kernel) so does the first; in the kernels
-  // of two transforms that spills 250 to 580 bytes at 64 registers.
+  // OPAQUE (four transforms in one kernel) so does the first.
   int t1 = t;
   if (OPAQUE) asm volatile("mov.b32 %0, %1;" : "=r"(t1) : "r"(t));
   line_dft<N>(v, tw, sm, t1);
@@ -125,13 +124,15 @@ __device__ __forceinline__ void af_load(float2 (&v)[kPointsPerThread], const AfA
 
 enum AfPass : int { kAfEntropy = 0, kAfAdjoint = 1, kAfRecompute = 2 };
 
-// Resident CTAs per SM: 64 registers (4 CTAs of 256 threads, 2 of 512) for the
-// entropy pass, as the compression lines; 128 for the gradient passes, whose
-// threads also keep the partial gradients of their pulses (more CTAs spill and
-// leave more partials to sum: 4 per SM 249 us a step, 2 per SM 224).
+// Resident CTAs per SM: two of 256 threads at 128 registers, one of 512.  More
+// do not help: the entropy pass takes 98 to 102 us a call at two, three or four
+// (its logarithms and transforms keep the issue slots 57 % busy), the adjoint
+// pass is slower at four (a step takes 249 us against 224) and leaves more
+// partial gradients to sum.  The number also fixes which rows a CTA's FP32
+// partial of the entropy adds up.
 template <int N, int PASS>
 constexpr int af_min_blocks() {
-  return PASS == kAfEntropy ? RowShape<N>::kMinBlocksDense : RowShape<N>::kThreads >= 512 ? 1 : 2;
+  return RowShape<N>::kThreads >= 512 ? 1 : 2;
 }
 
 template <int N, class TIn, int PASS>
