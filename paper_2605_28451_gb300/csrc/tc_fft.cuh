@@ -177,15 +177,26 @@ __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::aft
 // of the inverse takes bins j + 256 r, so the 16 results form row rho_0(j)
 // of A, four 16-byte stores.
 // The MMAs of one pass on the A tile as the CTA's threads left it: barrier,
-// four tcgen05.mma from one thread, commit, bounded wait.  Returns false
-// when the wait expired (all threads agree); after true the accumulators
-// may be read.
+// four tcgen05.mma from one thread, commit, bounded wait.  `meanwhile` runs
+// while they are in flight.  After the wait a thread may read the accumulators
+// and overwrite A at once: its own wait has seen the commit, so no second
+// barrier follows.  A wait that expires is kept in bit 31 of `phase`; the next
+// barrier makes it known to all threads, and the call returns false to all of
+// them (until then the thread works on with values that are not valid, as the
+// recorded timeout says).
+constexpr uint32_t kTcExpired = 0x80000000u;
+
+struct TcNothing {
+  __device__ __forceinline__ void operator()() const {}
+};
+
+template <class F = TcNothing>
 __device__ __forceinline__ bool tc_issue_wait(int* status, uint64_t* bar, uint32_t tmem, uint32_t a_base,
-                                              uint32_t b_base, uint32_t& phase) {
+                                              uint32_t b_base, uint32_t& phase, const F& meanwhile = F()) {
   using namespace tc;
   fence_proxy_async_shared();
   fence_before();
-  __syncthreads();
+  if (__syncthreads_or(int(phase & kTcExpired))) return false;
   if (threadIdx.x == 0) {
     fence_after();
 #pragma unroll
@@ -196,9 +207,10 @@ __device__ __forceinline__ bool tc_issue_wait(int* status, uint64_t* bar, uint32
                 tc::smem_desc(b_base + 2 * kLbo * s), s > 0);
     tc::commit(bar);
   }
-  const bool arrived = mbar_wait_bounded(bar, phase, status);
-  if (__syncthreads_or(!arrived)) return false;
+  meanwhile();
+  if (!mbar_wait_bounded(bar, phase & 1u, status)) phase |= kTcExpired;
   phase ^= 1;
+  __syncwarp();          // the reads of tensor memory that follow are warp-wide
   fence_after();
   return true;
 }
@@ -238,15 +250,15 @@ __device__ __forceinline__ void tc_filter_to_a(unsigned char* sA, int rho, const
 // in_scale * out_scale (one of them is 1), scales the first pass's results in
 // FP32 -- an exact power of two -- so the FP16 operands of the later passes
 // stay in range and the last pass writes the stored scale directly.
-template <int P, int MODE, bool FILTER = false, class TOut = __half2>
+template <int P, int MODE, bool FILTER = false, class TOut = __half2, class F = TcNothing>
 __device__ __forceinline__ bool tc_pass(const RowArgs& a, long long line, unsigned char* sA, uint64_t* bar,
                                         uint32_t tmem, uint32_t lane_tmem, uint32_t a_base, uint32_t b_base,
-                                        uint32_t& phase, const float2* s_tw) {
+                                        uint32_t& phase, const float2* s_tw, const F& meanwhile = F()) {
   using namespace tc;
   constexpr bool kFp8 = !std::is_same<TOut, __half2>::value;
   const int tid = threadIdx.x;
   const float sc = kFp8 && P == 0 ? a.in_scale * a.out_scale : 1.0f;
-  if (!tc_issue_wait(a.status, bar, tmem, a_base, b_base, phase)) return false;
+  if (!tc_issue_wait(a.status, bar, tmem, a_base, b_base, phase, meanwhile)) return false;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     uint32_t d[32];
@@ -365,13 +377,13 @@ __device__ __forceinline__ uint32_t tc_cta_setup(const void* tc_b, const float2*
   return *tslot;
 }
 
-// CTA teardown: a wait that expired leaves `phase` at the commit it was
-// waiting for; that commit gets one more bounded wait before the tensor
-// memory is freed.
+// CTA teardown: the commit of a wait that expired gets one more bounded wait
+// before the tensor memory is freed (`phase` has moved past it).
 __device__ __forceinline__ void tc_cta_teardown(bool ok, unsigned char* smem, uint32_t tmem, uint32_t phase) {
   using namespace tc;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kBarOff);
-  if (!ok && threadIdx.x == 0) mbar_wait_bounded(bar, phase, nullptr);
+  const bool expired = __syncthreads_or(int(!ok || (phase & kTcExpired) != 0u));
+  if (expired && threadIdx.x == 0) mbar_wait_bounded(bar, (phase & 1u) ^ 1u, nullptr);
   fence_before();
   __syncthreads();
   if ((threadIdx.x >> 5) == 0) {
@@ -382,7 +394,12 @@ __device__ __forceinline__ void tc_cta_teardown(bool ok, unsigned char* smem, ui
 // 128 threads per CTA, eight CTAs per SM: eight lines in flight per SM (the
 // TMEM limit at 64 columns a line) while each CTA's passes run one after
 // another.  Persistent: CTA b takes lines b, b + grid, ...; thread 0 bulk-
-// prefetches the CTA's next line into L2.
+// prefetches the CTA's next line into L2, and the first half of it may be
+// loaded while the last pass of the current one waits for its MMAs.  What
+// bounds it is that chain of passes (barrier, MMA, accumulator read, twiddles,
+// store), not DRAM: one barrier a pass instead of two took 32768 lines from
+// .2093 to .2054 ms and the compression of 8192 lines from .1129 to .1092, the
+// early loads the former to .2035 (5.28 TB/s).
 template <int MODE, class TIn, class TOut = __half2>
 __global__ void __launch_bounds__(tc::kThreads, tc::kCtasPerSm) fft_tc_kernel(const RowArgs a) {
   using namespace tc;
@@ -402,34 +419,46 @@ __global__ void __launch_bounds__(tc::kThreads, tc::kCtasPerSm) fft_tc_kernel(co
   uint32_t phase = 0;
   bool ok = true;
 
+  // Points j + 256 r, j = tid + 128 h, of a line as FP16 operands: complex64
+  // inputs are rounded here; FP8 pairs convert exactly.
+  auto load_half = [&](long long line, int h, uint32_t (&x)[16]) {
+    const TIn* in = in_lines + line * a.in_stride + tid + 128 * h;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      if constexpr (sizeof(TIn) == 4) {
+        x[r] = ld_once_b32(in + 256 * r);
+      } else if constexpr (sizeof(TIn) == 2) {
+        const __half2_raw v = __nv_cvt_fp8x2_to_halfraw2(__nv_fp8x2_storage_t(ld_once_b16(in + 256 * r)),
+                                                         Fp8Format<TIn>::kInterp);
+        x[r] = uint32_t(v.x) | (uint32_t(v.y) << 16);
+      } else {
+        const __half2 v = __float22half2_rn(ld_once_f2(in + 256 * r));
+        x[r] = *reinterpret_cast<const uint32_t*>(&v);
+      }
+    }
+  };
+  // The early loads hold 16 registers through the last pass: FP16 pairs of the
+  // plain transforms have them, the compression and the conversions of the
+  // other types would spill (e4m3 .209 -> .219 ms, compression .109 -> .113).
+  constexpr bool kEarly = MODE != kCompress && sizeof(TIn) == 4;
+  uint32_t first[16];
+  if (kEarly && (long long)blockIdx.x < a.lines) load_half(blockIdx.x, 0, first);
+
   for (long long line = blockIdx.x; ok && line < a.lines; line += gridDim.x) {
     const long long next = line + gridDim.x;
     if (a.pf_ahead > 0 && tid == 0 && next < a.lines)   // next iteration's line, into L2
       prefetch_l2_bulk(in_lines + next * a.in_stride, uint32_t(kN * sizeof(TIn)));
     // Pass-0 inputs: butterfly j takes x[j + 256 r]; its row of A is four
     // 16-byte core-matrix rows, one st.shared.v4 per four points (the eight
-    // lanes of a quarter-warp have distinct row % 8).  Complex64 inputs are
-    // rounded to FP16 operands here; FP8 pairs convert exactly.
-    const TIn* in = in_lines + line * a.in_stride + tid;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int j = tid + 128 * h;
-      uint32_t x[16];
-#pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        if constexpr (sizeof(TIn) == 4) {
-          x[r] = ld_once_b32(in + 128 * h + 256 * r);
-        } else if constexpr (sizeof(TIn) == 2) {
-          const __half2_raw v = __nv_cvt_fp8x2_to_halfraw2(
-              __nv_fp8x2_storage_t(ld_once_b16(in + 128 * h + 256 * r)), Fp8Format<TIn>::kInterp);
-          x[r] = uint32_t(v.x) | (uint32_t(v.y) << 16);
-        } else {
-          const __half2 v = __float22half2_rn(ld_once_f2(in + 128 * h + 256 * r));
-          x[r] = *reinterpret_cast<const uint32_t*>(&v);
-        }
-      }
-      tc_store_row0(sA, j, x);
-    }
+    // lanes of a quarter-warp have distinct row % 8).
+    if constexpr (!kEarly) load_half(line, 0, first);
+    tc_store_row0(sA, tid, first);
+    uint32_t second[16];
+    load_half(line, 1, second);
+    tc_store_row0(sA, tid + 128, second);
+    auto next_half = [&]() {
+      if (kEarly && next < a.lines) load_half(next, 0, first);
+    };
     if constexpr (MODE == kCompress) {
       // Forward, filter (into A, conjugated and shifted), inverse: the inverse's
       // input is already conj(Y) / N, so its first pass takes plain B.
@@ -438,11 +467,11 @@ __global__ void __launch_bounds__(tc::kThreads, tc::kCtasPerSm) fft_tc_kernel(co
            tc_pass<2, MODE, true>(a, line, sA, bar, tmem, lane_tmem, a_base, b_base, phase, s_tw) &&
            tc_pass<0, MODE>(a, line, sA, bar, tmem, lane_tmem, a_base, b_base, phase, s_tw) &&
            tc_pass<1, MODE>(a, line, sA, bar, tmem, lane_tmem, a_base, b_base, phase, s_tw) &&
-           tc_pass<2, MODE>(a, line, sA, bar, tmem, lane_tmem, a_base, b_last, phase, s_tw);
+           tc_pass<2, MODE, false, TOut>(a, line, sA, bar, tmem, lane_tmem, a_base, b_last, phase, s_tw, next_half);
     } else {
       ok = tc_pass<0, MODE, false, TOut>(a, line, sA, bar, tmem, lane_tmem, a_base, b_first, phase, s_tw) &&
            tc_pass<1, MODE, false, TOut>(a, line, sA, bar, tmem, lane_tmem, a_base, b_base, phase, s_tw) &&
-           tc_pass<2, MODE, false, TOut>(a, line, sA, bar, tmem, lane_tmem, a_base, b_last, phase, s_tw);
+           tc_pass<2, MODE, false, TOut>(a, line, sA, bar, tmem, lane_tmem, a_base, b_last, phase, s_tw, next_half);
     }
   }
   tc_cta_teardown(ok, smem_tc, tmem, phase);
