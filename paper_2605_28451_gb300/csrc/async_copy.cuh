@@ -34,6 +34,18 @@ __device__ __forceinline__ void check_finite(int* flag, F value) {
   note_nonfinite(flag, bad);
 }
 
+// First statement of a kernel that launch_chained starts: it may be running
+// while the kernel before it in the stream still is.  From the wait on, that
+// kernel is complete and its writes are visible, so every access to memory
+// that a kernel may have written comes after it (through coherent loads:
+// ld.global.nc would ask for data that nobody writes while the grid runs).
+// Only then is the next kernel let in, so at most one is ever waiting.  Both
+// instructions do nothing in an ordinary launch.
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(128, 3) fft_long_kernel(const RowArgs a) {
   constexpr float kInvN = 1.0f / float(N);
   extern __shared__ float4 smem_long[];
   __shared__ __align__(8) uint64_t bar;
+  chain_begin();
   float2* sm = reinterpret_cast<float2*>(smem_long);
   const int u = threadIdx.x;
   const int c = int(cooperative_groups::this_cluster().block_rank());
@@ -220,41 +221,17 @@ template <int N, class TS, int MODE, bool SCALED, bool H16ROW = false>
 cudaError_t launch_long_n(const RowArgs& a, cudaStream_t stream) {
   using S = LongShape<N>;
   auto kern = fft_long_kernel<N, TS, MODE, SCALED, H16ROW>;
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(S::kThreads);
-  cfg.dynamicSmemBytes = S::kSmemBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = S::C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  // One-time set-up (thread-safe, see setup_kernel): the shared-memory
-  // attribute and the number of resident clusters.
-  static const LaunchSetup setup = [&]() -> LaunchSetup {
-    LaunchSetup r{cudaSuccess, 0};
-    r.err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::kSmemBytes));
-    if (r.err != cudaSuccess) return r;
-    cudaLaunchConfig_t probe = cfg;
-    probe.gridDim = dim3(S::C);
-    r.err = cudaOccupancyMaxActiveClusters(&r.resident, kern, &probe);
-    return r;
-  }();
+  static const LaunchSetup setup = setup_cluster_kernel(kern, S::C, S::kThreads, S::kSmemBytes);
   if (setup.err != cudaSuccess) return setup.err;
   if (a.lines <= 0) return cudaSuccess;
   const long long grid = a.lines * S::C;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  cfg.gridDim = dim3(unsigned(grid));
   RowArgs b = a;
   b.pf_ahead = (a.variant == kRowsPlainL2 || a.variant == kRowsPlain4L2 || a.variant == kRowsPlainHL2 ||
                 a.variant == kRowsPlainH4L2 || a.variant == kRowsPlainHS4L2)
                    ? setup.resident
                    : 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, b);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_chained(kern, grid, S::kThreads, S::kSmemBytes, S::C, a.line_off == nullptr, stream, b);
 }
 
 }  // namespace bfp

@@ -58,6 +58,7 @@ __device__ __forceinline__ float2 unit_of(unsigned long long phase) {
 // cells; rate[r] for the n_rg range bins: k_a(R_r) / 2 turns.
 __global__ void rda_lines_kernel(RdaGeometry geo, int range_dependent, int n_az, int n_rg,
                                  unsigned long long* __restrict__ shift, unsigned long long* __restrict__ rate) {
+  chain_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n_az) {
     const int k = i < n_az / 2 ? i : i - n_az;
@@ -82,6 +83,7 @@ rda_rows_kernel(const RdaArgs a) {
   extern __shared__ float2 smem_rda[];
   __shared__ float warp_max[32];
   __shared__ float2 ramp[AZIMUTH ? 1 : G][P];
+  chain_begin();
   const int g = threadIdx.x / T;
   const int t = threadIdx.x - g * T;
   const long long line = (long long)blockIdx.x * G + g;
@@ -177,8 +179,7 @@ cudaError_t launch_rda_n(const RdaArgs& a, cudaStream_t s) {
   if (setup.err != cudaSuccess) return setup.err;
   if (a.lines <= 0) return cudaSuccess;
   const long long grid = (a.lines + S::G - 1) / S::G;
-  kern<<<dim3(unsigned(grid)), dim3(S::kThreads), S::kSmemBytes, s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, S::kThreads, S::kSmemBytes, 1, true, s, a);
 }
 
 template <class TS, bool AZIMUTH>
@@ -198,8 +199,8 @@ cudaError_t launch_rda_typed(int log2n, const RdaArgs& a, cudaStream_t s) {
 
 cudaError_t launch_rda_lines(const RdaGeometry& geo, bool range_dependent, int n_az, int n_rg,
                              unsigned long long* shift, unsigned long long* rate, cudaStream_t s) {
-  rda_lines_kernel<<<(n_az + n_rg + 127) / 128, 128, 0, s>>>(geo, range_dependent, n_az, n_rg, shift, rate);
-  return cudaGetLastError();
+  const long long grid = (n_az + n_rg + 127) / 128;
+  return launch_chained(rda_lines_kernel, grid, 128, 0, 1, true, s, geo, int(range_dependent), n_az, n_rg, shift, rate);
 }
 
 cudaError_t launch_rcmc_rows(int log2n, bool f16, const RdaArgs& a, cudaStream_t s) {

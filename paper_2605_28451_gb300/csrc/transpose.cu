@@ -36,7 +36,7 @@ struct TileIo {
     r0 = (b / col_tiles) * TILE;
   }
   // This thread's share of tile b: ROUNDS rows of VEC consecutive elements.
-  __device__ void load(const T* __restrict__ in, long long b, int lr, int rr, T (&e)[ROUNDS][VEC]) const {
+  __device__ void load(const T* in, long long b, int lr, int rr, T (&e)[ROUNDS][VEC]) const {
     long long r0, c0;
     origin(b, r0, c0);
     const bool vec = r0 + TILE <= rows && c0 + TILE <= cols && cols % VEC == 0;
@@ -56,12 +56,13 @@ struct TileIo {
 };
 
 template <class T>
-__global__ void __launch_bounds__(256, 8) transpose_kernel(const T* __restrict__ in, T* __restrict__ out,
+__global__ void __launch_bounds__(256, 8) transpose_kernel(const T* in, T* out,
                                                         long long rows, long long cols, long long col_tiles,
                                                         long long tiles) {
   using Io = TileIo<T>;
   constexpr int VEC = Io::VEC, TILE = Io::TILE, ROUNDS = Io::ROUNDS;
   __shared__ T tile[TILE][TILE + 1];
+  chain_begin();
   const Io io{rows, cols, col_tiles};
   const int lr = threadIdx.x % 16, rr = threadIdx.x / 16;
   long long b = blockIdx.x;
@@ -126,15 +127,11 @@ cudaError_t launch_transpose(const void* in, void* out, long long rows, long lon
   // Every CTA takes the same number of tiles (the last ones one fewer at most).
   const long long per_cta = (tiles + res - 1) / res;
   const long long grid = (tiles + per_cta - 1) / per_cta;
-  const dim3 block{256u, 1u, 1u};
-  if (elem_bytes == 4) {
-    transpose_kernel<unsigned int><<<unsigned(grid), block, 0, s>>>(
-        static_cast<const unsigned int*>(in), static_cast<unsigned int*>(out), rows, cols, gx, tiles);
-  } else {
-    transpose_kernel<float2><<<unsigned(grid), block, 0, s>>>(static_cast<const float2*>(in),
-                                                             static_cast<float2*>(out), rows, cols, gx, tiles);
-  }
-  return cudaGetLastError();
+  if (elem_bytes == 4)
+    return launch_chained(transpose_kernel<unsigned int>, grid, 256, 0, 1, true, s,
+                          static_cast<const unsigned int*>(in), static_cast<unsigned int*>(out), rows, cols, gx, tiles);
+  return launch_chained(transpose_kernel<float2>, grid, 256, 0, 1, true, s, static_cast<const float2*>(in),
+                        static_cast<float2*>(out), rows, cols, gx, tiles);
 }
 
 }  // namespace bfp

@@ -186,13 +186,13 @@ __device__ __forceinline__ void wide_filter(float2 (&v)[WideShape<N>::P], const 
   constexpr int kAhead = N <= 4096 ? 8 : 0;
   float2 w[2][8];
 #pragma unroll
-  for (int i = 0; i < kAhead; ++i) w[0][i] = __ldg(h + T * i);
+  for (int i = 0; i < kAhead; ++i) w[0][i] = h[T * i];
 #pragma unroll
   for (int m0 = 0; m0 < P; m0 += 8) {
     const int load = m0 + kAhead;
     if (load < P) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) w[(load / 8) & 1][i] = __ldg(h + T * (load + i));
+      for (int i = 0; i < 8; ++i) w[(load / 8) & 1][i] = h[T * (load + i)];
     }
     if (kAhead > 0) asm volatile("" ::: "memory");
 #pragma unroll
@@ -258,6 +258,7 @@ fft_wide_kernel(const RowArgs a) {
   constexpr bool kSplit = kWideSplit<N, MODE>;
   static_assert(kWideOffered<N, TIn, MODE>, "see kWideOffered");
   extern __shared__ float4 smem_wide[];
+  chain_begin();
   const int g = threadIdx.x / T;
   const int t = threadIdx.x - g * T;
   const long long line = (long long)blockIdx.x * G + g;
@@ -332,6 +333,7 @@ fft_wide_stream_kernel(const RowArgs a) {
   static_assert(N * sizeof(TIn) <= wide_line_floats<N, false>() * sizeof(float), "the line fits the exchange buffer");
   extern __shared__ float4 smem_wide[];
   __shared__ __align__(8) uint64_t bar;
+  chain_begin();
   float* sm = reinterpret_cast<float*>(smem_wide);
   auto issue = [&](long long l) {
     mbar_arrive_expect_tx(&bar, uint32_t(N * sizeof(TIn)));
@@ -389,8 +391,7 @@ cudaError_t launch_wide_n(const RowArgs& a, cudaStream_t stream, bool l2_prefetc
       if (setup.err != cudaSuccess) return setup.err;
       if (a.lines <= 0) return cudaSuccess;
       const int grid = int(a.lines < setup.resident ? a.lines : setup.resident);
-      kern<<<grid, S::kThreads, kBytes, stream>>>(a);
-      return cudaGetLastError();
+      return launch_chained(kern, grid, S::kThreads, kBytes, 1, a.line_off == nullptr, stream, a);
     }
   }
   constexpr size_t kBytes = size_t(S::G) * wide_line_floats<N, kWideSplit<N, MODE>>() * sizeof(float);
@@ -402,8 +403,7 @@ cudaError_t launch_wide_n(const RowArgs& a, cudaStream_t stream, bool l2_prefetc
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   RowArgs b = a;
   b.pf_ahead = l2_prefetch && a.in_stride == N ? setup.resident : 0;
-  kern<<<dim3(unsigned(grid)), dim3(S::kThreads), kBytes, stream>>>(b);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, S::kThreads, kBytes, 1, a.line_off == nullptr, stream, b);
 }
 
 }  // namespace bfp
