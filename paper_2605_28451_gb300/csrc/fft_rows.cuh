@@ -799,9 +799,11 @@ LaunchSetup setup_kernel(K kern, int threads, size_t smem) {
 // inverse: 256 points, 8 lines, 8.2 -> 6.4 us; 4096 points, 256 lines, 12.3 ->
 // 10.9; 1024 points, 30011 lines, 86.0 -> 81.6; a SAR image of 4096 x 4096
 // (four kernels) 183 -> 176; with migration correction (nine) 335 -> 318.
-// `chained` is false where other streams' kernels would use the places that
-// the waiting CTAs hold: the listed lines of a ragged batch, one stream per
-// length (20000 lines: 773 us chained, 768 not).
+// A ragged batch, two streams with one kernel per length: 2000 lines 105.6 ->
+// 96.6 us in FP16, 20000 lines 900 -> 877 us in FP32; in FP16 20000 lines take
+// 788 -> 784 us alone and 769 -> 774 in a stream of such calls, whose waiting
+// CTAs hold places that the other stream's kernels would use.
+// `chained` is false where it measured slower (launch_tc_kernel).
 // `cluster`: CTAs per thread-block cluster.
 template <class K, class... A>
 cudaError_t launch_chained(K kern, long long grid, int threads, size_t smem, int cluster, bool chained,
@@ -1171,7 +1173,7 @@ cudaError_t launch_fourstep_n(const RowArgs& a, cudaStream_t stream) {
                 a.variant == kRowsPlainH4L2 || a.variant == kRowsPlainHS4L2)
                    ? resident_clusters
                    : 0;
-  return launch_chained(kern, grid, 256, kBytes, N1, a.line_off == nullptr, stream, b);
+  return launch_chained(kern, grid, 256, kBytes, N1, true, stream, b);
 }
 
 // Lines longer than one CTA's share (N >= 8192): a line spans a thread-block
@@ -1261,7 +1263,7 @@ cudaError_t launch_rows_plain_x(const RowArgs& a, cudaStream_t stream, bool l2_p
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   RowArgs b = a;
   b.pf_ahead = l2_prefetch ? resident : 0;
-  return launch_chained(kern, grid, S::kThreads, kBytes, 1, a.line_off == nullptr, stream, b);
+  return launch_chained(kern, grid, S::kThreads, kBytes, 1, true, stream, b);
 }
 
 }  // namespace bfp
@@ -1368,7 +1370,7 @@ cudaError_t launch_rows_n(const RowArgs& a, cudaStream_t stream) {
   const bool l2 = a.variant == kRowsPlainL2 || a.variant == kRowsPlain4L2 || a.variant == kRowsPlainHL2 ||
                   a.variant == kRowsPlainH4L2 || a.variant == kRowsPlainHS4L2;
   b.pf_ahead = (l2 && !TLOAD && a.in_stride == N) ? resident : 0;
-  return launch_chained(kern, grid, S::kThreads, kBytes, S::C, a.line_off == nullptr, stream, b);
+  return launch_chained(kern, grid, S::kThreads, kBytes, S::C, true, stream, b);
   }
 }
 

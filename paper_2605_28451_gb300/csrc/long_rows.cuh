@@ -231,7 +231,7 @@ cudaError_t launch_long_n(const RowArgs& a, cudaStream_t stream) {
                 a.variant == kRowsPlainH4L2 || a.variant == kRowsPlainHS4L2)
                    ? setup.resident
                    : 0;
-  return launch_chained(kern, grid, S::kThreads, S::kSmemBytes, S::C, a.line_off == nullptr, stream, b);
+  return launch_chained(kern, grid, S::kThreads, S::kSmemBytes, S::C, true, stream, b);
 }
 
 }  // namespace bfp

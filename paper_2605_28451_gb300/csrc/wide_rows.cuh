@@ -391,7 +391,7 @@ cudaError_t launch_wide_n(const RowArgs& a, cudaStream_t stream, bool l2_prefetc
       if (setup.err != cudaSuccess) return setup.err;
       if (a.lines <= 0) return cudaSuccess;
       const int grid = int(a.lines < setup.resident ? a.lines : setup.resident);
-      return launch_chained(kern, grid, S::kThreads, kBytes, 1, a.line_off == nullptr, stream, a);
+      return launch_chained(kern, grid, S::kThreads, kBytes, 1, true, stream, a);
     }
   }
   constexpr size_t kBytes = size_t(S::G) * wide_line_floats<N, kWideSplit<N, MODE>>() * sizeof(float);
@@ -403,7 +403,7 @@ cudaError_t launch_wide_n(const RowArgs& a, cudaStream_t stream, bool l2_prefetc
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   RowArgs b = a;
   b.pf_ahead = l2_prefetch && a.in_stride == N ? setup.resident : 0;
-  return launch_chained(kern, grid, S::kThreads, kBytes, 1, a.line_off == nullptr, stream, b);
+  return launch_chained(kern, grid, S::kThreads, kBytes, 1, true, stream, b);
 }
 
 }  // namespace bfp

@@ -96,6 +96,34 @@ def test_dependent_transforms(n, lines, storage, arith):
         assert B.bfpfft_plan_status(p) == B.OK
 
 
+@pytest.mark.parametrize("count", [40, 1500])
+@pytest.mark.parametrize("storage", [B.F16_BFP, B.F32])
+def test_dependent_ragged_batches(count, storage):
+    """Per-length kernels on the caller's stream and the plan's own, each exec reading what the last one wrote."""
+    import torch
+    n = synth.uneven_lengths(count, seed=count)
+    off = n.cumsum() - n
+    start = noise((int(n.sum()), 2), count)
+    start = start.half() if storage == B.F16_BFP else torch.view_as_complex(start)
+    plans = [B.bfpfft_plan_create_many(n, off, storage, d) for d in (B.FORWARD, B.INVERSE)]
+    for p in plans:
+        B.bfpfft_plan_set_many_schedule(p, 0, B.MANY_PER_LENGTH)
+    own = [start.clone(), torch.zeros_like(start), torch.zeros_like(start)]
+
+    def reset():
+        own[0].copy_(start)
+        own[1].zero_()
+        own[2].zero_()
+
+    expect = run_chain(plans, own, True).clone()
+    for _ in range(3):
+        reset()
+        assert torch.equal(run_chain(plans, own, False), expect)
+    assert torch.equal(run_captured(lambda: run_chain(plans, own, False), reset), expect)
+    for p in plans:
+        assert B.bfpfft_plan_status(p) == B.OK
+
+
 @pytest.mark.parametrize("n_az,n_rg", [(512, 256), (256, 1024), (1024, 2048)])
 @pytest.mark.parametrize("out", [B.F16_BFP, B.F32])
 def test_filter_made_and_used_in_one_chain(n_az, n_rg, out):
