@@ -770,9 +770,10 @@ def _bench_uneven(B, torch, dev, stream):
         plan = B.bfpfft_plan_create_many(lengths, offsets, dtype, B.FORWARD)
         # The tuner's pick among cluster counts, two-pass long lines, one launch
         # per length and (FP16 exchanges allowed) the FP16 row exchange of
-        # four-step lines; one FP16 plan keeps the untuned persistent kernel.
+        # long lines; one FP16 plan runs the persistent kernel.
         if name == "f16_bfp_persistent_kernel":
             code = 0
+            B.bfpfft_plan_set_many_schedule(plan, 0, 0)
         else:
             code, _ = B.bfpfft_plan_tune(plan, allow_fp16_exchange=name == "f16_bfp_tuned_fp16_exchange")
         for _ in range(3):
