@@ -62,6 +62,7 @@ fft_rows_adaptive_kernel(const RowArgs a) {
   constexpr int P = S::P, T = S::T, G = S::G;
   extern __shared__ float2 smem_ad[];
   __shared__ uint32_t warp_max[32];
+  chain_begin();
   const int g = threadIdx.x / T;
   const int t = threadIdx.x - g * T;
   const long long line = (long long)blockIdx.x * G + g;
@@ -133,8 +134,7 @@ cudaError_t launch_adaptive_n(const RowArgs& a, cudaStream_t stream) {
   // Dense rows in device memory: each CTA prefetches the lines of the CTA one
   // resident wave later into L2 (as the default row variant does).
   b.pf_ahead = (a.no_prefetch || a.in_stride != N) ? 0 : setup.resident;
-  kern<<<dim3(unsigned(grid)), dim3(S::kThreads), S::kSmemBytes, stream>>>(b);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, S::kThreads, S::kSmemBytes, 1, true, stream, b);
 }
 
 // Dispatch on log2 N in [4, 14] (lines held by one CTA).

@@ -273,6 +273,7 @@ fft_rows16_kernel(const RowArgs a) {
   using A = A16<H>;
   constexpr int P = S::P, T = S::T, G = S::G;
   extern __shared__ uint32_t smem16[];
+  chain_begin();
   const int g = threadIdx.x / T;
   const int t = threadIdx.x - g * T;
   const long long line = (long long)blockIdx.x * G + g;
@@ -317,7 +318,7 @@ fft_rows16_kernel(const RowArgs a) {
     for (int m0 = 0; m0 < P; m0 += 4) {
       float2 h[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) h[i] = __ldg(a.h + (active ? line : 0) * a.h_stride + t + T * (m0 + i));
+      for (int i = 0; i < 4; ++i) h[i] = a.h[(active ? line : 0) * a.h_stride + t + T * (m0 + i)];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const H w = A::make(h[i].x, h[i].y), wp = A::make(-h[i].y, h[i].x);
@@ -354,8 +355,7 @@ cudaError_t launch_rows16_nl(const RowArgs& a, cudaStream_t stream) {
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   RowArgs b = a;
   b.pf_ahead = (a.no_prefetch || a.in_stride != N) ? 0 : setup.resident;
-  kern<<<dim3(unsigned(grid)), dim3(S::kThreads), kBytes, stream>>>(b);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, S::kThreads, kBytes, 1, true, stream, b);
 }
 
 // Exchange layout kPadQ (the swizzle and plain pad32 measured the same time as

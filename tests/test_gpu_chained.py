@@ -66,16 +66,21 @@ SHAPES = [(16, 40), (256, 8), (512, 300), (1024, 77), (2048, 1300), (4096, 100),
 
 
 @pytest.mark.parametrize("n,lines", SHAPES)
-@pytest.mark.parametrize("storage,arith", [(B.F16_BFP, None), (B.F32, None), (B.F16_BFP, "tc")])
-def test_dependent_transforms(n, lines, storage, arith):
+@pytest.mark.parametrize("storage,arith", [(B.F16_BFP, None), (B.F32, None), (B.F16_BFP, "tc"), (B.F16_BFP, "f16"),
+                                           (B.BF16, None), (B.F16_BFP, "tma")])
+def test_dependent_transforms(n, lines, storage, arith, monkeypatch):
     import torch
     if arith == "tc" and n != 4096:
         pytest.skip("4096 points only")
+    if n > 16384 and (arith == "f16" or storage == B.BF16):
+        pytest.skip("16-bit arithmetic up to 16384 points")
+    if arith == "tma":
+        monkeypatch.setenv("BFPFFT_ROWS", "tma")
     start = noise((lines, n, 2), n + lines)
-    start = start.half() if storage == B.F16_BFP else torch.view_as_complex(start)
+    start = {B.F16_BFP: start.half(), B.BF16: start.bfloat16()}.get(storage, torch.view_as_complex(start))
     plans = [B.bfpfft_plan_create(n, lines, storage, d) for d in (B.FORWARD, B.INVERSE)]
-    for p in plans if arith else ():
-        B.bfpfft_plan_set_arith(p, B.ARITH_F16_MUL_F32_ACC)
+    for p in plans if arith in ("tc", "f16") else ():
+        B.bfpfft_plan_set_arith(p, B.ARITH_F16 if arith == "f16" else B.ARITH_F16_MUL_F32_ACC)
 
     def bufs():
         return [start.clone(), torch.zeros_like(start), torch.zeros_like(start)]
@@ -98,8 +103,10 @@ def test_dependent_transforms(n, lines, storage, arith):
 
 @pytest.mark.parametrize("count", [40, 1500])
 @pytest.mark.parametrize("storage", [B.F16_BFP, B.F32])
-def test_dependent_ragged_batches(count, storage):
-    """Per-length kernels on the caller's stream and the plan's own, each exec reading what the last one wrote."""
+@pytest.mark.parametrize("flags", [0, B.MANY_PER_LENGTH])
+def test_dependent_ragged_batches(count, storage, flags):
+    """The persistent kernel, or per-length kernels on the caller's stream and the plan's own, each exec reading what the
+    last one wrote."""
     import torch
     n = synth.uneven_lengths(count, seed=count)
     off = n.cumsum() - n
@@ -107,7 +114,7 @@ def test_dependent_ragged_batches(count, storage):
     start = start.half() if storage == B.F16_BFP else torch.view_as_complex(start)
     plans = [B.bfpfft_plan_create_many(n, off, storage, d) for d in (B.FORWARD, B.INVERSE)]
     for p in plans:
-        B.bfpfft_plan_set_many_schedule(p, 0, B.MANY_PER_LENGTH)
+        B.bfpfft_plan_set_many_schedule(p, 0, flags)
     own = [start.clone(), torch.zeros_like(start), torch.zeros_like(start)]
 
     def reset():
@@ -122,6 +129,27 @@ def test_dependent_ragged_batches(count, storage):
     assert torch.equal(run_captured(lambda: run_chain(plans, own, False), reset), expect)
     for p in plans:
         assert B.bfpfft_plan_status(p) == B.OK
+
+
+@pytest.mark.parametrize("n,lines", [(256, 30), (4096, 200), (16384, 40)])
+def test_adaptive_exponents_in_one_chain(n, lines):
+    """Mantissas and exponents written by one kernel are the next one's input."""
+    import torch
+    start = noise((lines, n, 2), n).half()
+    plans = [B.bfpfft_plan_create(n, lines, B.F16_ADAPTIVE, d) for d in (B.FORWARD, B.INVERSE)]
+    results = []
+    for between in (True, False, False):
+        x = [start.clone(), torch.zeros_like(start)]
+        e = [torch.full((lines,), 3, dtype=torch.int32, device="cuda:0"), torch.zeros(lines, dtype=torch.int32,
+                                                                                      device="cuda:0")]
+        for k in range(STEPS):
+            B.bfpfft_exec_adaptive(plans[k % 2], x[k % 2], e[k % 2], x[(k + 1) % 2], e[(k + 1) % 2])
+            if between:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        results.append((x[0], e[0]))
+    for x, e in results[1:]:
+        assert torch.equal(x, results[0][0]) and torch.equal(e, results[0][1])
 
 
 @pytest.mark.parametrize("n_az,n_rg", [(512, 256), (256, 1024), (1024, 2048)])
