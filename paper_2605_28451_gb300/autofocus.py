@@ -74,11 +74,15 @@ class SarEntropy(torch.autograd.Function):
         grad = torch.empty(n_az, dtype=torch.float32, device=phi_c.device)
         if kept and ws.arith == B.ARITH_F32 and ctx.versions == (rc._version, ha._version):
             state = kept[0]
-            B.sar_autofocus_grad_kept(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, state, state.numel(), g_e, grad,
+            B.sar_autofocus_grad_kept(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, state, state.numel(), None, grad,
                                       ws.stats, ws.buf, ws.bytes)
-            return grad, None, None, None, None, None
-        B.sar_autofocus_grad(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, grad, ws.stats, ws.buf, ws.bytes, arith=ws.arith)
-        return (g_e.to(torch.float32) * grad), None, None, None, None, None
+        else:
+            B.sar_autofocus_grad(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, grad, ws.stats, ws.buf, ws.bytes,
+                                 arith=ws.arith)
+        # A torch product, not the library's scale argument: g_e may carry a graph
+        # (create_graph), a batch (is_grads_batched) or a tangent (forward mode),
+        # which a raw pointer would lose.  g_e is a scalar: the product is FP32.
+        return g_e * grad, None, None, None, None, None
 
 
 def entropy(phi, rc, ha, rc_dtype: int, ws: Workspace):

@@ -1,0 +1,95 @@
+"""What the autofocus wrapper does around the library calls, with those replaced by a stand-in on the CPU whose entropy
+is linear, E = sum c phi with c = sum over the range bins of rc: the gradient is c times the upstream gradient exactly."""
+
+import ctypes
+
+import pytest
+import torch
+
+from paper_2605_28451_gb300 import autofocus as GA
+from paper_2605_28451_gb300 import bfpfft as B
+
+N_AZ, N_RG = 8, 3
+
+
+def column_sums(rc):
+    return rc.sum(0)
+
+
+class Library:
+    """The calls SarEntropy makes, and which of them were made."""
+
+    def __init__(self, monkeypatch):
+        self.calls = []
+        monkeypatch.setattr(B, "sar_autofocus_workspace_bytes", lambda n_az: 64)
+        monkeypatch.setattr(B, "sar_autofocus_state_bytes", lambda n_az, n_rg: 256 + 8 * n_az)
+        for name in ("entropy", "entropy_keep", "grad", "grad_kept"):
+            monkeypatch.setattr(B, "sar_autofocus_" + name, getattr(self, name))
+
+    def entropy(self, rc, rc_dtype, phi, ha, n_az, n_rg, stats, ws, ws_bytes, arith=B.ARITH_F32, stream=None):
+        self.calls.append("entropy")
+        stats[2] = (column_sums(rc) * phi).sum()
+
+    def entropy_keep(self, rc, rc_dtype, phi, ha, n_az, n_rg, stats, e, state, state_bytes, ws, ws_bytes, stream=None):
+        self.calls.append("entropy_keep")
+        e.copy_((column_sums(rc) * phi).sum())
+        state[:4 * n_az].view(torch.float32).copy_(column_sums(rc))
+
+    def grad(self, rc, rc_dtype, phi, ha, n_az, n_rg, grad, stats, ws, ws_bytes, arith=B.ARITH_F32, stream=None):
+        self.calls.append("grad")
+        grad.copy_(column_sums(rc))
+
+    def grad_kept(self, rc, rc_dtype, phi, ha, n_az, n_rg, state, state_bytes, scale, grad, stats, ws, ws_bytes,
+                  stream=None):
+        self.calls.append("grad_kept")
+        grad.copy_(state[:4 * n_az].view(torch.float32))
+        if scale is not None:   # the library reads it through its address
+            grad.mul_(ctypes.c_double.from_address(scale.data_ptr()).value)
+
+
+@pytest.fixture
+def library(monkeypatch):
+    return Library(monkeypatch)
+
+
+def scene(seed=0):
+    g = torch.Generator().manual_seed(seed)
+    rc = torch.randint(-4, 5, (N_RG, N_AZ), generator=g).float()
+    phi = torch.randint(-4, 5, (N_AZ,), generator=g).float().requires_grad_(True)
+    return rc, torch.ones(N_AZ), phi, GA.Workspace(N_AZ, "cpu")
+
+
+def test_gradient_stays_differentiable_in_the_upstream_gradient(library):
+    rc, ha, phi, ws = scene()
+    w = torch.tensor(3.0, dtype=torch.float64, requires_grad=True)
+    grad, = torch.autograd.grad(w * GA.entropy(phi, rc, ha, B.F32, ws), phi, create_graph=True)
+    assert library.calls == ["entropy_keep", "grad_kept"]
+    assert grad.dtype == torch.float32 and torch.equal(grad, 3.0 * column_sums(rc))
+    dw, = torch.autograd.grad(grad.sum(), w)
+    assert dw == column_sums(rc).sum()
+
+
+def test_directional_derivative(library):
+    rc, ha, phi, ws = scene(1)
+    v = torch.arange(1.0, N_AZ + 1)
+    _, d = torch.autograd.functional.jvp(lambda p: GA.entropy(p, rc, ha, B.F32, ws), phi.detach(), v)
+    assert d == (column_sums(rc) * v).sum()
+
+
+def test_batched_upstream_gradients(library):
+    rc, ha, phi, ws = scene(2)
+    e = GA.entropy(phi, rc, ha, B.F32, ws)
+    up = torch.tensor([1.0, -2.0, 5.0], dtype=torch.float64)
+    grad, = torch.autograd.grad(e, phi, grad_outputs=up, is_grads_batched=True)
+    assert grad.dtype == torch.float32 and torch.equal(grad, up.float()[:, None] * column_sums(rc))
+
+
+def test_tangent_of_the_upstream_gradient(library):
+    rc, ha, phi, ws = scene(3)
+    e = GA.entropy(phi, rc, ha, B.F32, ws)
+    with torch.autograd.forward_ad.dual_level():
+        up = torch.autograd.forward_ad.make_dual(torch.tensor(2.0, dtype=torch.float64),
+                                                 torch.tensor(7.0, dtype=torch.float64))
+        grad, = torch.autograd.grad(e, phi, grad_outputs=up)
+        primal, tangent = torch.autograd.forward_ad.unpack_dual(grad)
+    assert torch.equal(primal, 2.0 * column_sums(rc)) and torch.equal(tangent, 7.0 * column_sums(rc))
