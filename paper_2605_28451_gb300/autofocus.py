@@ -34,6 +34,14 @@ class Workspace:
 KEEP_BYTES = 512 << 20   # largest state kept between forward and backward
 
 
+def _versions(*tensors):
+    """The tensors' version counters, or None where one has none to tell a change
+    by (made under inference_mode, or not torch's)."""
+    if any(not isinstance(x, torch.Tensor) or x.is_inference() for x in tensors):
+        return None
+    return tuple(x._version for x in tensors)
+
+
 class SarEntropy(torch.autograd.Function):
     """E = entropy(|A(rc . exp(-j phi))|^2); d E / d phi by the GPU adjoint.
 
@@ -48,7 +56,8 @@ class SarEntropy(torch.autograd.Function):
         n_rg, n_az = rc.shape[0], rc.shape[1]
         phi_c = phi.detach().contiguous()
         ctx.rc, ctx.ha, ctx.rc_dtype, ctx.ws = rc, ha, rc_dtype, ws
-        if keep and ws.arith == B.ARITH_F32 and n_rg > 0:
+        versions = _versions(rc, ha) if keep and ws.arith == B.ARITH_F32 and n_rg > 0 else None
+        if versions is not None:
             size = B.sar_autofocus_state_bytes(n_az, n_rg)
             if 0 < size <= KEEP_BYTES:
                 try:
@@ -60,7 +69,7 @@ class SarEntropy(torch.autograd.Function):
                     B.sar_autofocus_entropy_keep(rc, rc_dtype, phi_c, ha, n_az, n_rg, ws.stats, e, state, size,
                                                  ws.buf, ws.bytes)
                     ctx.save_for_backward(phi_c, state)
-                    ctx.versions = (rc._version, ha._version)
+                    ctx.versions = versions
                     return e
         B.sar_autofocus_entropy(rc, rc_dtype, phi_c, ha, n_az, n_rg, ws.stats, ws.buf, ws.bytes, arith=ws.arith)
         ctx.save_for_backward(phi_c)
@@ -72,7 +81,7 @@ class SarEntropy(torch.autograd.Function):
         rc, ha, ws = ctx.rc, ctx.ha, ctx.ws
         n_rg, n_az = rc.shape[0], rc.shape[1]
         grad = torch.empty(n_az, dtype=torch.float32, device=phi_c.device)
-        if kept and ws.arith == B.ARITH_F32 and ctx.versions == (rc._version, ha._version):
+        if kept and ws.arith == B.ARITH_F32 and ctx.versions == _versions(rc, ha):
             state = kept[0]
             B.sar_autofocus_grad_kept(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, state, state.numel(), None, grad,
                                       ws.stats, ws.buf, ws.bytes)

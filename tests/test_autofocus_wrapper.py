@@ -93,3 +93,13 @@ def test_tangent_of_the_upstream_gradient(library):
         grad, = torch.autograd.grad(e, phi, grad_outputs=up)
         primal, tangent = torch.autograd.forward_ad.unpack_dual(grad)
     assert torch.equal(primal, 2.0 * column_sums(rc)) and torch.equal(tangent, 7.0 * column_sums(rc))
+
+
+@pytest.mark.parametrize("which", ["rc", "ha"])
+def test_inference_mode_tensors_are_accepted(library, which):
+    rc, ha, phi, ws = scene(4)
+    with torch.inference_mode():
+        rc, ha = (rc.clone(), ha) if which == "rc" else (rc, ha.clone())
+    grad, = torch.autograd.grad(GA.entropy(phi, rc, ha, B.F32, ws), phi)
+    assert torch.equal(grad, column_sums(rc))
+    assert library.calls == ["entropy", "grad"]   # no version counter to watch: nothing is kept
