@@ -5,7 +5,7 @@ phase-corrected data.  When a gradient will be asked for it also keeps the
 FP32 image (up to KEEP_BYTES) for backward, which then runs the hand-written
 adjoint alone: four transforms per range bin for a step instead of eight.
 Without the image (evaluation only, larger scenes, no memory for it, the
-tensor-core mode, rc or ha changed in place in between) backward calls
+tensor-core mode, saved-tensor hooks, rc or ha changed in place in between) backward calls
 ``sar_autofocus_grad``, which computes it again.  Only argument marshalling
 happens here.
 """
@@ -42,6 +42,14 @@ def _versions(*tensors):
     return tuple(x._version for x in tensors)
 
 
+def _saved_tensor_hooks() -> bool:
+    """Whether saved tensors pass through hooks (offloading, compression,
+    checkpointing).  Those are meant for saved inputs: the image, computed again
+    in a fraction of the time that moving it takes, is not handed to them."""
+    top = getattr(torch._C._autograd, "_top_saved_tensors_default_hooks", None)
+    return top is not None and top(False) is not None
+
+
 class SarEntropy(torch.autograd.Function):
     """E = entropy(|A(rc . exp(-j phi))|^2); d E / d phi by the GPU adjoint.
 
@@ -56,7 +64,8 @@ class SarEntropy(torch.autograd.Function):
         n_rg, n_az = rc.shape[0], rc.shape[1]
         phi_c = phi.detach().contiguous()
         ctx.rc, ctx.ha, ctx.rc_dtype, ctx.ws = rc, ha, rc_dtype, ws
-        versions = _versions(rc, ha) if keep and ws.arith == B.ARITH_F32 and n_rg > 0 else None
+        keep = keep and ws.arith == B.ARITH_F32 and n_rg > 0 and not _saved_tensor_hooks()
+        versions = _versions(rc, ha) if keep else None
         if versions is not None:
             size = B.sar_autofocus_state_bytes(n_az, n_rg)
             if 0 < size <= KEEP_BYTES:

@@ -103,3 +103,17 @@ def test_inference_mode_tensors_are_accepted(library, which):
     grad, = torch.autograd.grad(GA.entropy(phi, rc, ha, B.F32, ws), phi)
     assert torch.equal(grad, column_sums(rc))
     assert library.calls == ["entropy", "grad"]   # no version counter to watch: nothing is kept
+
+
+def test_saved_tensor_hooks_see_the_phase_only(library):
+    rc, ha, phi, ws = scene(5)
+    seen = []
+
+    def pack(x):
+        seen.append(x)
+        return x.half()
+    with torch.autograd.graph.saved_tensors_hooks(pack, lambda x: x.float()):
+        e = GA.entropy(phi, rc, ha, B.F32, ws)
+    grad, = torch.autograd.grad(e, phi)
+    assert len(seen) == 1 and torch.equal(seen[0], phi.detach())
+    assert torch.equal(grad, column_sums(rc)) and library.calls == ["entropy", "grad"]
