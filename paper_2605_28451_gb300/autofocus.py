@@ -5,9 +5,13 @@ phase-corrected data.  When a gradient will be asked for it also keeps the
 FP32 image (up to KEEP_BYTES) for backward, which then runs the hand-written
 adjoint alone: four transforms per range bin for a step instead of eight.
 Without the image (evaluation only, larger scenes, no memory for it, the
-tensor-core mode, saved-tensor hooks, rc or ha changed in place in between) backward calls
-``sar_autofocus_grad``, which computes it again.  Only argument marshalling
-happens here.
+tensor-core mode, saved-tensor hooks, rc or ha written in between) backward
+calls ``sar_autofocus_grad``, which computes it again.  A write is seen by the
+tensors' version counters: torch's own operations and this package's calls
+advance them.  Where something else writes rc or ha (another library's kernel,
+a replayed CUDA graph, a call given a bare address), it must advance them too
+(``torch.autograd.graph.increment_version``) or wait until backward has run.
+Only argument marshalling happens here.
 """
 
 from __future__ import annotations

@@ -2,8 +2,9 @@
 
 Argument marshalling only: every function here converts torch tensors to raw
 device pointers and the current CUDA stream, calls the C entry point of the
-same name, and turns a non-zero status into ``BfpfftError``.  There is no
-fallback: if the compiled library is missing, the first call raises.
+same name, and turns a non-zero status into ``BfpfftError``.  Output tensors'
+version counters advance as after torch's own in-place operations.  There is
+no fallback: if the compiled library is missing, the first call raises.
 """
 
 from __future__ import annotations
@@ -147,9 +148,29 @@ def error_string(status: int) -> str:
         return "unknown"
 
 
-def _check(status: int, where: str):
+def _check(status: int, where: str, *written):
+    """Raise for a non-zero status; else mark the arrays that the call wrote."""
     if status != OK:
         raise BfpfftError(status, where)
+    if written:
+        _mark_written(written)
+
+
+_tensor = _increment_version = None
+
+
+def _mark_written(arrays):
+    """Advance the version counters of the torch tensors among `arrays`, as torch's
+    own in-place operations do: autograd then sees that a tensor which it (or
+    the autofocus wrapper) holds was rewritten through its address."""
+    global _tensor, _increment_version
+    if _tensor is None:
+        import torch
+        _increment_version = torch.autograd.graph.increment_version
+        _tensor = torch.Tensor
+    for x in arrays:
+        if isinstance(x, _tensor):
+            _increment_version(x)
 
 
 def _ptr(x) -> int | None:
@@ -211,7 +232,7 @@ def bfpfft_plan_create(n: int, batch: int, dtype: int, direction: int) -> Plan:
 
 
 def bfpfft_exec(plan: Plan, inp, out, stream=None):
-    _check(lib().bfpfft_exec(plan.handle, _ptr(inp), _ptr(out), _stream(stream)), "bfpfft_exec")
+    _check(lib().bfpfft_exec(plan.handle, _ptr(inp), _ptr(out), _stream(stream)), "bfpfft_exec", out)
 
 
 def bfpfft_plan_create_many(n, offset_pts, dtype: int, direction: int) -> Plan:
@@ -243,7 +264,7 @@ def bfpfft_plan_tune(plan: Plan, allow_fp16_exchange: bool = False):
 
 
 def bfpfft_exec_graph(plan: Plan, inp, out, stream=None):
-    _check(lib().bfpfft_exec_graph(plan.handle, _ptr(inp), _ptr(out), _stream(stream)), "bfpfft_exec_graph")
+    _check(lib().bfpfft_exec_graph(plan.handle, _ptr(inp), _ptr(out), _stream(stream)), "bfpfft_exec_graph", out)
 
 
 def bfpfft_plan_destroy(plan: Plan):
@@ -293,49 +314,49 @@ def bfpfft_plan_selftest_wait(plan: Plan, stream=None):
 def bfpfft_exec_adaptive(plan: Plan, inp, in_exp, out, out_exp, stream=None):
     """FP16 mantissas + int32 per-line exponents in and out (in_exp may be None)."""
     _check(lib().bfpfft_exec_adaptive(plan.handle, _ptr(inp), _ptr(in_exp), _ptr(out), _ptr(out_exp),
-                                      _stream(stream)), "bfpfft_exec_adaptive")
+                                      _stream(stream)), "bfpfft_exec_adaptive", out, out_exp)
 
 
 def bfp_spectral_filter(x, x_dtype: int, h, h_stride: int, out, out_dtype: int, n: int, lines: int,
                         arith: int = ARITH_F32, stream=None):
     _check(lib().bfp_spectral_filter(_ptr(x), int(x_dtype), _ptr(h), int(h_stride), _ptr(out), int(out_dtype), int(n),
-                                     int(lines), int(arith), _stream(stream)), "bfp_spectral_filter")
+                                     int(lines), int(arith), _stream(stream)), "bfp_spectral_filter", out)
 
 
 def bfp_spectral_adaptive(x, x_dtype: int, x_exp, h, out, out_exp, n: int, lines: int, stream=None):
     _check(lib().bfp_spectral_adaptive(_ptr(x), int(x_dtype), _ptr(x_exp), _ptr(h), _ptr(out), _ptr(out_exp),
-                                       int(n), int(lines), _stream(stream)), "bfp_spectral_adaptive")
+                                       int(n), int(lines), _stream(stream)), "bfp_spectral_adaptive", out, out_exp)
 
 
 def sar_make_filter(ref, n: int, peak_normalise: bool, h_out, stream=None):
     _check(lib().sar_make_filter(_ptr(ref), int(n), int(bool(peak_normalise)), _ptr(h_out), _stream(stream)),
-           "sar_make_filter")
+           "sar_make_filter", h_out)
 
 
 def sar_range_compress(raw, raw_dtype: int, out, out_dtype: int, hr, n_az: int, n_rg: int,
                        transpose_out: bool = False, stream=None):
     _check(lib().sar_range_compress(_ptr(raw), int(raw_dtype), _ptr(out), int(out_dtype), _ptr(hr), int(n_az),
-                                    int(n_rg), int(bool(transpose_out)), _stream(stream)), "sar_range_compress")
+                                    int(n_rg), int(bool(transpose_out)), _stream(stream)), "sar_range_compress", out)
 
 
 def sar_azimuth_compress(rc, rc_dtype: int, rc_layout: int, img, img_dtype: int, ha, n_az: int, n_rg: int,
                          stream=None):
     _check(lib().sar_azimuth_compress(_ptr(rc), int(rc_dtype), int(rc_layout), _ptr(img), int(img_dtype), _ptr(ha),
-                                      int(n_az), int(n_rg), _stream(stream)), "sar_azimuth_compress")
+                                      int(n_az), int(n_rg), _stream(stream)), "sar_azimuth_compress", img)
 
 
 def sar_range_compress_arith(raw, raw_dtype: int, out, out_dtype: int, hr, n_az: int, n_rg: int,
                              transpose_out: bool, arith: int, stream=None):
     _check(lib().sar_range_compress_arith(_ptr(raw), int(raw_dtype), _ptr(out), int(out_dtype), _ptr(hr), int(n_az),
                                           int(n_rg), int(bool(transpose_out)), int(arith), _stream(stream)),
-           "sar_range_compress_arith")
+           "sar_range_compress_arith", out)
 
 
 def sar_azimuth_compress_arith(rc, rc_dtype: int, rc_layout: int, img, img_dtype: int, ha, n_az: int, n_rg: int,
                                arith: int, stream=None):
     _check(lib().sar_azimuth_compress_arith(_ptr(rc), int(rc_dtype), int(rc_layout), _ptr(img), int(img_dtype),
                                             _ptr(ha), int(n_az), int(n_rg), int(arith), _stream(stream)),
-           "sar_azimuth_compress_arith")
+           "sar_azimuth_compress_arith", img)
 
 
 RDA_RCMC = 1
@@ -348,7 +369,7 @@ def sar_rda_image(raw, raw_dtype: int, img, img_dtype: int, hr, n_az: int, n_rg:
     """geometry: (range cell m, PRF Hz, wavelength m, speed m/s, centre slant range m)."""
     g = (ctypes.c_double * 5)(*[float(v) for v in geometry])
     _check(lib().sar_rda_image(_ptr(raw), int(raw_dtype), _ptr(img), int(img_dtype), _ptr(hr), int(n_az), int(n_rg),
-                               ctypes.cast(g, _vp), int(aperture), int(flags), _stream(stream)), "sar_rda_image")
+                               ctypes.cast(g, _vp), int(aperture), int(flags), _stream(stream)), "sar_rda_image", img)
 
 
 def bfp_sqnr_workspace_bytes() -> int:
@@ -358,7 +379,7 @@ def bfp_sqnr_workspace_bytes() -> int:
 def bfp_sqnr_sums(ref, ref_dtype: int, test, test_dtype: int, count: int, sums_out, workspace, ws_bytes: int,
                   stream=None):
     _check(lib().bfp_sqnr_sums(_ptr(ref), int(ref_dtype), _ptr(test), int(test_dtype), int(count), _ptr(sums_out),
-                               _ptr(workspace), int(ws_bytes), _stream(stream)), "bfp_sqnr_sums")
+                               _ptr(workspace), int(ws_bytes), _stream(stream)), "bfp_sqnr_sums", sums_out)
 
 
 def sqnr_from_sums(s) -> dict:
@@ -382,14 +403,14 @@ def sar_autofocus_entropy(rc, rc_dtype: int, phi, ha, n_az: int, n_rg: int, stat
                           stream=None, arith: int = ARITH_F32):
     _check(lib().sar_autofocus_entropy_arith(_ptr(rc), int(rc_dtype), _ptr(phi), _ptr(ha), int(n_az), int(n_rg),
                                              _ptr(stats_out), _ptr(workspace), int(ws_bytes), int(arith),
-                                             _stream(stream)), "sar_autofocus_entropy")
+                                             _stream(stream)), "sar_autofocus_entropy", stats_out)
 
 
 def sar_autofocus_grad(rc, rc_dtype: int, phi, ha, n_az: int, n_rg: int, grad_out, stats_out, workspace,
                        ws_bytes: int, stream=None, arith: int = ARITH_F32):
     _check(lib().sar_autofocus_grad_arith(_ptr(rc), int(rc_dtype), _ptr(phi), _ptr(ha), int(n_az), int(n_rg),
                                           _ptr(grad_out), _ptr(stats_out), _ptr(workspace), int(ws_bytes),
-                                          int(arith), _stream(stream)), "sar_autofocus_grad")
+                                          int(arith), _stream(stream)), "sar_autofocus_grad", grad_out, stats_out)
 
 
 def sar_autofocus_state_bytes(n_az: int, n_rg: int) -> int:
@@ -402,7 +423,7 @@ def sar_autofocus_entropy_keep(rc, rc_dtype: int, phi, ha, n_az: int, n_rg: int,
     _check(lib().sar_autofocus_entropy_keep(_ptr(rc), int(rc_dtype), _ptr(phi), _ptr(ha), int(n_az), int(n_rg),
                                             _ptr(stats_out), _ptr(entropy_out), _ptr(state), int(state_bytes),
                                             _ptr(workspace), int(ws_bytes), _stream(stream)),
-           "sar_autofocus_entropy_keep")
+           "sar_autofocus_entropy_keep", stats_out, entropy_out, state)
 
 
 def sar_autofocus_grad_kept(rc, rc_dtype: int, phi, ha, n_az: int, n_rg: int, state, state_bytes: int, scale,
@@ -410,7 +431,7 @@ def sar_autofocus_grad_kept(rc, rc_dtype: int, phi, ha, n_az: int, n_rg: int, st
     _check(lib().sar_autofocus_grad_kept(_ptr(rc), int(rc_dtype), _ptr(phi), _ptr(ha), int(n_az), int(n_rg),
                                          _ptr(state), int(state_bytes), _ptr(scale), _ptr(grad_out),
                                          _ptr(stats_out), _ptr(workspace), int(ws_bytes), _stream(stream)),
-           "sar_autofocus_grad_kept")
+           "sar_autofocus_grad_kept", grad_out, stats_out)
 
 
 def bfp_sqnr_sums_noalloc_max_count() -> int:
@@ -420,7 +441,7 @@ def bfp_sqnr_sums_noalloc_max_count() -> int:
 def bfp_sqnr_sums_noalloc(ref, ref_dtype: int, test, test_dtype: int, count: int, sums_out, stream=None):
     """bfp_sqnr_sums with the library's built-in scratch: no workspace, no allocation."""
     _check(lib().bfp_sqnr_sums_noalloc(_ptr(ref), int(ref_dtype), _ptr(test), int(test_dtype), int(count),
-                                       _ptr(sums_out), _stream(stream)), "bfp_sqnr_sums_noalloc")
+                                       _ptr(sums_out), _stream(stream)), "bfp_sqnr_sums_noalloc", sums_out)
 
 
 PT_FIELDS = ("pslr_range_db", "pslr_azimuth_db", "islr_range_db", "islr_azimuth_db", "width_range_cells",
@@ -435,4 +456,4 @@ def sar_point_target_metrics(img, img_dtype: int, n_az: int, n_rg: int, targets,
                              ws_bytes: int, stream=None):
     _check(lib().sar_point_target_metrics(_ptr(img), int(img_dtype), int(n_az), int(n_rg), _ptr(targets), int(k),
                                           int(guard), _ptr(out), _ptr(workspace), int(ws_bytes), _stream(stream)),
-           "sar_point_target_metrics")
+           "sar_point_target_metrics", out)

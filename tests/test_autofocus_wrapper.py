@@ -117,3 +117,46 @@ def test_saved_tensor_hooks_see_the_phase_only(library):
     grad, = torch.autograd.grad(e, phi)
     assert len(seen) == 1 and torch.equal(seen[0], phi.detach())
     assert torch.equal(grad, column_sums(rc)) and library.calls == ["entropy", "grad"]
+
+
+def test_scene_and_filter_refilled_by_the_library(library, monkeypatch):
+    class Refill:
+        """Writes its output through the address it gets, as the compiled library does."""
+
+        def __getattr__(self, name):
+            def call(*args):
+                out = {"sar_range_compress": 2, "bfpfft_exec": 2, "sar_make_filter": 3}[name]
+                ctypes.memmove(args[out], new.data_ptr(), new.numel() * 4)
+                return B.OK
+            return call
+    monkeypatch.setattr(B, "lib", Refill)
+    for case in ("range", "exec", "filter"):
+        rc, ha, phi, ws = scene(6)
+        new = scene(7)[0] if case != "filter" else ha.clone()
+        e = GA.entropy(phi, rc, ha, B.F32, ws)
+        if case == "range":
+            B.sar_range_compress(new, B.F32, rc, B.F32, ha, N_RG, N_AZ, stream=0)
+        elif case == "exec":
+            B.bfpfft_exec(B.Plan(None, N_AZ, N_RG, B.F32, B.FORWARD), new, rc, stream=0)
+        else:
+            B.sar_make_filter(new, N_AZ, False, ha, stream=0)
+        grad, = torch.autograd.grad(e, phi)
+        assert torch.equal(grad, column_sums(rc)), case
+        assert library.calls[-1] == "grad", case
+
+
+def test_only_calls_that_succeed_mark_their_outputs(monkeypatch):
+    status = B.OK
+    monkeypatch.setattr(B, "lib", lambda: type("Lib", (), {"bfpfft_exec": staticmethod(lambda *a: status),
+                                                           "bfpfft_error_string": staticmethod(lambda s: b"")}))
+    plan = B.Plan(None, 16, 1, B.F32, B.FORWARD)
+    x, y = torch.zeros(16), torch.zeros(16)
+    B.bfpfft_exec(plan, x, y, stream=0)
+    assert (x._version, y._version) == (0, 1)
+    B.bfpfft_exec(plan, x.data_ptr(), y.data_ptr(), stream=0)      # addresses: nothing to mark
+    with torch.inference_mode():
+        B.bfpfft_exec(plan, x, torch.zeros(16), stream=0)          # no counter to advance
+    status = B.ERR_MISALIGNED
+    with pytest.raises(B.BfpfftError):
+        B.bfpfft_exec(plan, x, y, stream=0)
+    assert y._version == 1
