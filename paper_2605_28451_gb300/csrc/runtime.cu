@@ -632,8 +632,10 @@ extern "C" int bfpfft_exec(bfpfft_plan plan, const void* in, void* out, void* st
 // kernel cannot use because its CTAs are sized for every length at once.
 // With FP8 storage each length keeps the block exponents of its uniform plan.
 // Lines of 32768 / 65536 points run on the caller's stream, the shorter
-// lengths on the plan's side stream forked from it (an event each way, so a
-// stream capture takes both branches), so that their launches overlap.
+// lengths on the plan's side stream forked from it (an event each way), so that
+// their launches overlap.  Inside a stream capture everything stays on the
+// caller's stream: the side stream would belong to that capture until it ends,
+// and any other call on the plan would meet it there.
 static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStream_t s) {
   std::lock_guard<std::mutex> lock(plan->fork_mutex);   // host threads may share a plan
   const bool dev_mem = device_memory(in);
@@ -641,7 +643,10 @@ static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStre
   bool has_long = false, has_short = false;
   for (int l = kMinLog2; l <= kMaxLog2; ++l)
     if (plan->len_count[l] > 0) (l >= 15 ? has_long : has_short) = true;
-  const bool fork = has_long && has_short && plan->side != nullptr;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t ce = cudaStreamIsCapturing(s, &capture);
+  if (ce != cudaSuccess) return cuda_status(ce);
+  const bool fork = has_long && has_short && plan->side != nullptr && capture == cudaStreamCaptureStatusNone;
   if (fork) {
     cudaError_t e = cudaEventRecord(plan->ev_fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(plan->side, plan->ev_fork, 0);
@@ -676,7 +681,7 @@ static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStre
     }
     if (e != cudaSuccess) result = cuda_status(e);
   }
-  if (fork) {   // joined whatever happened, so that a capture stays well formed
+  if (fork) {   // joined whatever happened: the shorter lengths are work of the caller's stream
     cudaError_t e = cudaEventRecord(plan->ev_join, plan->side);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, plan->ev_join, 0);
     if (e != cudaSuccess && result == BFPFFT_OK) result = cuda_status(e);
