@@ -470,6 +470,15 @@ __global__ void conj_normalise_kernel(float2* h, int n, int peak_normalise) {
 
 }  // namespace
 
+// A side stream with the events that fork it from the caller's stream and join
+// it back.
+struct Fork {
+  cudaStream_t side = nullptr;
+  cudaEvent_t out = nullptr;
+  cudaEvent_t back = nullptr;
+};
+constexpr int kMaxForks = 8;   // of one plan
+
 struct bfpfft_plan_s {
   int64_t n;
   int64_t batch;
@@ -498,14 +507,13 @@ struct bfpfft_plan_s {
   int per_length = -1;                  // one dense-row launch per length over its listed lines (1), the persistent
                                         // kernel (0), or by the batch's size (-1, see large_batch)
   bool large_batch = false;             // at least kPerLengthPoints points
-  std::mutex fork_mutex;                // the side stream and the two events below serve one exec at a time
+  std::mutex fork_mutex;                // the forks below serve one exec at a time
   int has_fourstep = 0;                 // some line has 8192 points or more
   long long len_first[kMaxLog2 + 1] = {};   // lines of 2^l points: first index into d_line_off ...
   long long len_count[kMaxLog2 + 1] = {};   // ... and count
   const float2* tw_len[kMaxLog2 + 1] = {};  // per-length twiddle tables (device pointers, shared cache)
-  cudaStream_t side = nullptr;          // one launch per length: the shorter lengths' stream (owned) ...
-  cudaEvent_t ev_fork = nullptr;        // ... forked from the caller's stream ...
-  cudaEvent_t ev_join = nullptr;        // ... and joined back into it
+  Fork forks[kMaxForks];                // one launch per length: streams for the shorter lengths (owned) ...
+  int num_forks = 0;                    // ... of which made so far
   int first_short_task = 0;             // first task of a length below 32768
   long long long_first[2] = {0, 0};     // lines of 65536 / 32768 points: first index into d_line_off ...
   long long long_count[2] = {0, 0};     // ... and count
@@ -533,6 +541,23 @@ namespace {
 // 16 ... 1024: 2.8 M 20 / 29, 6.9 M 30 / 34).
 constexpr int64_t kPerLengthPoints = int64_t(1) << 23;
 
+void destroy_fork(Fork* f) {
+  if (f->side) cudaStreamDestroy(f->side);
+  if (f->out) cudaEventDestroy(f->out);
+  if (f->back) cudaEventDestroy(f->back);
+}
+
+cudaError_t create_fork(Fork* f) {
+  cudaError_t e = cudaStreamCreateWithFlags(&f->side, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f->out, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f->back, cudaEventDisableTiming);
+  if (e != cudaSuccess) {
+    destroy_fork(f);
+    *f = Fork{};
+  }
+  return e;
+}
+
 void free_plan_resources(bfpfft_plan p) {
   if (p->graph) cudaGraphExecDestroy(p->graph);
   if (p->status) cudaFree(p->status);
@@ -540,9 +565,36 @@ void free_plan_resources(bfpfft_plan p) {
   if (p->d_tasks) cudaFree(p->d_tasks);
   if (p->d_tw) cudaFree(p->d_tw);
   if (p->d_tw4) cudaFree(p->d_tw4);
-  if (p->side) cudaStreamDestroy(p->side);
-  if (p->ev_fork) cudaEventDestroy(p->ev_fork);
-  if (p->ev_join) cudaEventDestroy(p->ev_join);
+  for (int i = 0; i < p->num_forks; ++i) destroy_fork(&p->forks[i]);
+}
+
+// The fork for an execution on `s`.  A side stream that a stream capture has
+// taken in belongs to that capture until it ends, so eager executions and every
+// open capture of the plan get one each, made when first needed (in relaxed
+// capture mode, as it may be inside a capture) and used again afterwards.  Null:
+// none to be had, or kMaxForks in open captures; everything stays on `s` then.
+Fork* pick_fork(bfpfft_plan p, cudaStream_t s) {
+  cudaStreamCaptureStatus mine, its;
+  unsigned long long my_id = 0, its_id = 0;
+  cudaError_t e = cudaStreamGetCaptureInfo(s, &mine, &my_id);
+  for (int i = 0; i < p->num_forks && e == cudaSuccess; ++i) {
+    e = cudaStreamGetCaptureInfo(p->forks[i].side, &its, &its_id);
+    if (e == cudaSuccess &&
+        (its == cudaStreamCaptureStatusNone ||
+         (its == cudaStreamCaptureStatusActive && mine == cudaStreamCaptureStatusActive && its_id == my_id)))
+      return &p->forks[i];
+  }
+  if (e == cudaSuccess && p->num_forks < kMaxForks) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) {
+      e = create_fork(&p->forks[p->num_forks]);
+      cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    if (e == cudaSuccess) return &p->forks[p->num_forks++];
+  }
+  if (e != cudaSuccess) (void)cudaGetLastError();   // not an error of the launches that follow
+  return nullptr;
 }
 
 // The plan's status word: one device int, zeroed.
@@ -632,10 +684,8 @@ extern "C" int bfpfft_exec(bfpfft_plan plan, const void* in, void* out, void* st
 // kernel cannot use because its CTAs are sized for every length at once.
 // With FP8 storage each length keeps the block exponents of its uniform plan.
 // Lines of 32768 / 65536 points run on the caller's stream, the shorter
-// lengths on the plan's side stream forked from it (an event each way), so that
-// their launches overlap.  Inside a stream capture everything stays on the
-// caller's stream: the side stream would belong to that capture until it ends,
-// and any other call on the plan would meet it there.
+// lengths on a side stream of the plan forked from it (pick_fork), so that their
+// launches overlap.
 static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStream_t s) {
   std::lock_guard<std::mutex> lock(plan->fork_mutex);   // host threads may share a plan
   const bool dev_mem = device_memory(in);
@@ -643,19 +693,16 @@ static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStre
   bool has_long = false, has_short = false;
   for (int l = kMinLog2; l <= kMaxLog2; ++l)
     if (plan->len_count[l] > 0) (l >= 15 ? has_long : has_short) = true;
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  cudaError_t ce = cudaStreamIsCapturing(s, &capture);
-  if (ce != cudaSuccess) return cuda_status(ce);
-  const bool fork = has_long && has_short && plan->side != nullptr && capture == cudaStreamCaptureStatusNone;
+  const Fork* fork = has_long && has_short ? pick_fork(plan, s) : nullptr;
   if (fork) {
-    cudaError_t e = cudaEventRecord(plan->ev_fork, s);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(plan->side, plan->ev_fork, 0);
+    cudaError_t e = cudaEventRecord(fork->out, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(fork->side, fork->out, 0);
     if (e != cudaSuccess) return cuda_status(e);
   }
   int result = BFPFFT_OK;
   for (int l = kMaxLog2; l >= kMinLog2 && result == BFPFFT_OK; --l) {
     if (plan->len_count[l] == 0) continue;
-    const cudaStream_t ls = fork && l < 15 ? plan->side : s;
+    const cudaStream_t ls = fork && l < 15 ? fork->side : s;
     bfp::RowArgs a{};
     a.in = in;
     a.out = out;
@@ -681,9 +728,9 @@ static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStre
     }
     if (e != cudaSuccess) result = cuda_status(e);
   }
-  if (fork) {   // joined whatever happened: the shorter lengths are work of the caller's stream
-    cudaError_t e = cudaEventRecord(plan->ev_join, plan->side);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, plan->ev_join, 0);
+  if (fork) {   // joined whatever happened, so that a capture stays well formed
+    cudaError_t e = cudaEventRecord(fork->back, fork->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, fork->back, 0);
     if (e != cudaSuccess && result == BFPFFT_OK) result = cuda_status(e);
   }
   return result;
@@ -1154,9 +1201,8 @@ int bfpfft_plan_create_many(bfpfft_plan* out, int64_t count, const int64_t* n, c
     if (e == cudaSuccess) e = cudaMemcpy(p->d_tw, tw_host, sizeof(tw_host), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_tw4, tw4_host, sizeof(tw4_host), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = bfp::uneven_max_clusters(kind, direction == BFPFFT_INVERSE, &p->clusters);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = create_fork(&p->forks[0]);
+    if (e == cudaSuccess) p->num_forks = 1;
     if (e != cudaSuccess) st = cuda_status(e);
     if (st == BFPFFT_OK && p->clusters <= 0) st = BFPFFT_ERR_UNSUPPORTED;
   }

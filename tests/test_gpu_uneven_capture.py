@@ -61,3 +61,34 @@ def test_executed_while_captured(threads):
     torch.cuda.synchronize()
     assert torch.equal(captured, twice)
     assert B.bfpfft_plan_status(plan) == B.OK
+
+
+def test_two_captures_open_at_once():
+    """Each capture forks onto a stream of its own; an execution after both takes either again."""
+    import torch
+    plan, xs, expect = plan_and_data()
+    outs, graphs = [torch.zeros_like(x) for x in xs], [torch.cuda.CUDAGraph() for _ in xs]
+    first, second = torch.cuda.Stream(), torch.cuda.Stream()
+    opened, done = threading.Event(), threading.Event()
+
+    def hold_open():
+        with torch.cuda.graph(graphs[1], stream=second, capture_error_mode="thread_local"):
+            B.bfpfft_exec(plan, xs[1], outs[1])
+            opened.set()
+            done.wait(60)
+            B.bfpfft_exec(plan, xs[1], outs[1])
+    torch.cuda.synchronize()
+    t = threading.Thread(target=hold_open)
+    t.start()
+    assert opened.wait(60)
+    B.bfpfft_exec_graph(plan, xs[0], outs[0], stream=first)      # captures by itself, then replays
+    done.set()
+    t.join()
+    graphs[1].replay()
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0], expect[0]) and torch.equal(outs[1], expect[1])
+    eager = torch.zeros_like(xs[0])
+    B.bfpfft_exec(plan, xs[0], eager)
+    torch.cuda.synchronize()
+    assert torch.equal(eager, expect[0])
+    assert B.bfpfft_plan_status(plan) == B.OK
