@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 
 from . import build as _build
 
@@ -148,36 +149,37 @@ def error_string(status: int) -> str:
         return "unknown"
 
 
+_tensor = ()                # torch.Tensor, from the first one on
+_increment_version = None
+
+
+def _meet_torch():
+    """Called for an argument that may be the first torch tensor."""
+    global _tensor, _increment_version
+    torch = sys.modules.get("torch")
+    if torch is not None and _increment_version is None:
+        _increment_version = getattr(torch._C, "_increment_version", torch.autograd.graph.increment_version)
+        _tensor = torch.Tensor
+
+
 def _check(status: int, where: str, *written):
-    """Raise for a non-zero status; else mark the arrays that the call wrote."""
+    """Raise for a non-zero status.  Else advance the version counters of the torch
+    tensors that the call wrote, as torch's own in-place operations do: autograd
+    (and the autofocus wrapper) then sees that a tensor it holds was rewritten
+    through its address."""
     if status != OK:
         raise BfpfftError(status, where)
-    if written:
-        _mark_written(written)
-
-
-_tensor = _increment_version = None
-
-
-def _mark_written(arrays):
-    """Advance the version counters of the torch tensors among `arrays`, as torch's
-    own in-place operations do: autograd then sees that a tensor which it (or
-    the autofocus wrapper) holds was rewritten through its address."""
-    global _tensor, _increment_version
-    if _tensor is None:
-        import torch
-        _increment_version = torch.autograd.graph.increment_version
-        _tensor = torch.Tensor
-    for x in arrays:
+    for x in written:
         if isinstance(x, _tensor):
-            _increment_version(x)
+            _increment_version((x,))
 
 
 def _ptr(x) -> int | None:
-    if x is None:
-        return None
-    if isinstance(x, int):
+    if isinstance(x, _tensor):
+        return x.data_ptr()
+    if x is None or isinstance(x, int):
         return x
+    _meet_torch()
     return x.data_ptr()
 
 
@@ -232,7 +234,15 @@ def bfpfft_plan_create(n: int, batch: int, dtype: int, direction: int) -> Plan:
 
 
 def bfpfft_exec(plan: Plan, inp, out, stream=None):
-    _check(lib().bfpfft_exec(plan.handle, _ptr(inp), _ptr(out), _stream(stream)), "bfpfft_exec", out)
+    # As every other call here, but written out: the shortest transforms take the
+    # GPU less time than the helpers take the host.
+    status = (_lib or lib()).bfpfft_exec(plan.handle, inp.data_ptr() if isinstance(inp, _tensor) else _ptr(inp),
+                                         out.data_ptr() if isinstance(out, _tensor) else _ptr(out),
+                                         _current_stream() if stream is None and _current_stream else _stream(stream))
+    if status != OK:
+        raise BfpfftError(status, "bfpfft_exec")
+    if isinstance(out, _tensor):
+        _increment_version((out,))
 
 
 def bfpfft_plan_create_many(n, offset_pts, dtype: int, direction: int) -> Plan:

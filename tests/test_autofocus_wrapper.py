@@ -129,7 +129,7 @@ def test_scene_and_filter_refilled_by_the_library(library, monkeypatch):
                 ctypes.memmove(args[out], new.data_ptr(), new.numel() * 4)
                 return B.OK
             return call
-    monkeypatch.setattr(B, "lib", Refill)
+    monkeypatch.setattr(B, "_lib", Refill())
     for case in ("range", "exec", "filter"):
         rc, ha, phi, ws = scene(6)
         new = scene(7)[0] if case != "filter" else ha.clone()
@@ -147,8 +147,8 @@ def test_scene_and_filter_refilled_by_the_library(library, monkeypatch):
 
 def test_only_calls_that_succeed_mark_their_outputs(monkeypatch):
     status = B.OK
-    monkeypatch.setattr(B, "lib", lambda: type("Lib", (), {"bfpfft_exec": staticmethod(lambda *a: status),
-                                                           "bfpfft_error_string": staticmethod(lambda s: b"")}))
+    monkeypatch.setattr(B, "_lib", type("Lib", (), {"bfpfft_exec": staticmethod(lambda *a: status),
+                                                    "bfpfft_error_string": staticmethod(lambda s: b"")}))
     plan = B.Plan(None, 16, 1, B.F32, B.FORWARD)
     x, y = torch.zeros(16), torch.zeros(16)
     B.bfpfft_exec(plan, x, y, stream=0)
