@@ -95,9 +95,9 @@ __device__ __forceinline__ void dft4(float2& a0, float2& a1, float2& a2, float2&
   a3 = csub(t1, e);
 }
 
-template <int R> struct Dft;
+template <int R, bool FINE = false> struct Dft;
 
-template <> struct Dft<2> {
+template <bool FINE> struct Dft<2, FINE> {
   __device__ __forceinline__ static void run(float2 (&v)[2]) {
     const float2 a = v[0], b = v[1];
     v[0] = cadd(a, b);
@@ -105,7 +105,7 @@ template <> struct Dft<2> {
   }
 };
 
-template <> struct Dft<4> {
+template <bool FINE> struct Dft<4, FINE> {
   __device__ __forceinline__ static void run(float2 (&v)[4]) { dft4(v[0], v[1], v[2], v[3]); }
 };
 
@@ -132,7 +132,7 @@ __device__ __forceinline__ float2 sub_r2(float2 a, float2 b) {
 
 // 8 = 2 x 4: r = r1 + 2 r2, k = k2 + 4 k1.  The odd half's W8 and W8^3 have
 // their sqrt(1/2) folded into the last butterflies.
-template <> struct Dft<8> {
+template <bool FINE> struct Dft<8, FINE> {
   __device__ __forceinline__ static void run(float2 (&v)[8]) {
     dft4(v[0], v[2], v[4], v[6]);           // r1 = 0 -> a0[k2] at v[0,2,4,6]
     dft4(v[1], v[3], v[5], v[7]);           // r1 = 1 -> a1[k2] at v[1,3,5,7]
@@ -147,7 +147,7 @@ template <> struct Dft<8> {
 };
 
 // 16 = 4 x 4: r = r1 + 4 r2, k = k2 + 4 k1.
-template <> struct Dft<16> {
+template <bool FINE> struct Dft<16, FINE> {
   __device__ __forceinline__ static void run(float2 (&v)[16]) {
 #pragma unroll
     for (int r1 = 0; r1 < 4; ++r1) dft4(v[r1], v[r1 + 4], v[r1 + 8], v[r1 + 12]);
@@ -206,8 +206,16 @@ __host__ __device__ constexpr double cos_turn(int e, int m) {
 __host__ __device__ constexpr double sin_turn(int e, int m) { return cos_turn((e + 3 * m / 4) % m, m); }   // cos(x - pi / 2)
 
 // a * W_M^E = a * exp(-2 pi i E / M); the eighth roots cost two to four
-// instructions less than a full product.
-template <int E, int M>
+// instructions less than a full product.  cos(pi / 16) and cos(pi / 8) happen to
+// lie almost half an FP32 step (0.499 and 0.475) from their rounded values, and
+// every line takes the same few constants, so their errors add up: FINE, for
+// results stored in FP32, adds the low part of the constant that is further off,
+// at two multiplies a product.  Relative L2 error of FP32 lines in passes of radix
+// 16, in these radices without the low parts, and with them (1e-7): 1024 points
+// 1.083, 1.107, 1.031; 16384 1.326, 1.351, 1.267; 32768 1.378, 1.431, 1.354;
+// 65536 1.449, 1.473, 1.402.  It costs 1 to 2 % of the time from 8192 points on
+// (2^26 points: 16384 221.6 -> 223.9 us, 65536 251.5 -> 257.6), none below.
+template <int E, int M, bool FINE>
 __device__ __forceinline__ float2 mul_root(float2 a) {
   constexpr int e = E % M;
   if constexpr (e == 0) return a;
@@ -215,43 +223,48 @@ __device__ __forceinline__ float2 mul_root(float2 a) {
   else if constexpr (8 * e == M) return mul_w16_2(a);
   else if constexpr (8 * e == 3 * M) return mul_w16_6(a);
   else {
-    constexpr float c = float(cos_turn(e, M)), s = float(-sin_turn(e, M));
-    return cmul(a, make_float2(c, s));
+    constexpr double cd = cos_turn(e, M), sd = -sin_turn(e, M);
+    constexpr float c = float(cd), s = float(sd), cl = float(cd - double(c)), sl = float(sd - double(s));
+    if constexpr (!FINE) return cmul(a, make_float2(c, s));
+    else if constexpr (cl * cl >= sl * sl)
+      return make_float2(fmaf(a.x, c, fmaf(-a.y, s, a.x * cl)), fmaf(a.x, s, fmaf(a.y, c, a.y * cl)));
+    else
+      return make_float2(fmaf(a.x, c, fmaf(-a.y, s, -a.y * sl)), fmaf(a.x, s, fmaf(a.y, c, a.x * sl)));
   }
 }
 
 // v[k2] *= W_M^(R1 k2) for the eight k2.
-template <int R1, int M>
+template <int R1, int M, bool FINE>
 __device__ __forceinline__ void mul_roots8(float2 (&v)[8]) {
-  v[1] = mul_root<R1, M>(v[1]);
-  v[2] = mul_root<2 * R1, M>(v[2]);
-  v[3] = mul_root<3 * R1, M>(v[3]);
-  v[4] = mul_root<4 * R1, M>(v[4]);
-  v[5] = mul_root<5 * R1, M>(v[5]);
-  v[6] = mul_root<6 * R1, M>(v[6]);
-  v[7] = mul_root<7 * R1, M>(v[7]);
+  v[1] = mul_root<R1, M, FINE>(v[1]);
+  v[2] = mul_root<2 * R1, M, FINE>(v[2]);
+  v[3] = mul_root<3 * R1, M, FINE>(v[3]);
+  v[4] = mul_root<4 * R1, M, FINE>(v[4]);
+  v[5] = mul_root<5 * R1, M, FINE>(v[5]);
+  v[6] = mul_root<6 * R1, M, FINE>(v[6]);
+  v[7] = mul_root<7 * R1, M, FINE>(v[7]);
 }
 
 // Column r1 of an R1 x 8 split: the 8-point DFT of v[r1 + R1 r2] over r2,
 // times W_M^(r1 k2), back in place at v[r1 + R1 k2].
-template <int r1, int R1, int M>
+template <int r1, int R1, bool FINE, int M>
 __device__ __forceinline__ void dft8_column(float2 (&v)[M]) {
   float2 u[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) u[i] = v[r1 + R1 * i];
   Dft<8>::run(u);
-  mul_roots8<r1, M>(u);
+  mul_roots8<r1, M, FINE>(u);
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[r1 + R1 * i] = u[i];
 }
 
 // 32 = 4 x 8: r = r1 + 4 r2, k = k2 + 8 k1.
-template <> struct Dft<32> {
+template <bool FINE> struct Dft<32, FINE> {
   __device__ __forceinline__ static void run(float2 (&v)[32]) {
-    dft8_column<0, 4>(v);
-    dft8_column<1, 4>(v);
-    dft8_column<2, 4>(v);
-    dft8_column<3, 4>(v);
+    dft8_column<0, 4, FINE>(v);
+    dft8_column<1, 4, FINE>(v);
+    dft8_column<2, 4, FINE>(v);
+    dft8_column<3, 4, FINE>(v);
     float2 o[32];
 #pragma unroll
     for (int k2 = 0; k2 < 8; ++k2) {
@@ -268,16 +281,16 @@ template <> struct Dft<32> {
 };
 
 // 64 = 8 x 8: r = r1 + 8 r2, k = k2 + 8 k1.
-template <> struct Dft<64> {
+template <bool FINE> struct Dft<64, FINE> {
   __device__ __forceinline__ static void run(float2 (&v)[64]) {
-    dft8_column<0, 8>(v);
-    dft8_column<1, 8>(v);
-    dft8_column<2, 8>(v);
-    dft8_column<3, 8>(v);
-    dft8_column<4, 8>(v);
-    dft8_column<5, 8>(v);
-    dft8_column<6, 8>(v);
-    dft8_column<7, 8>(v);
+    dft8_column<0, 8, FINE>(v);
+    dft8_column<1, 8, FINE>(v);
+    dft8_column<2, 8, FINE>(v);
+    dft8_column<3, 8, FINE>(v);
+    dft8_column<4, 8, FINE>(v);
+    dft8_column<5, 8, FINE>(v);
+    dft8_column<6, 8, FINE>(v);
+    dft8_column<7, 8, FINE>(v);
     float2 o[64];
 #pragma unroll
     for (int k2 = 0; k2 < 8; ++k2) {

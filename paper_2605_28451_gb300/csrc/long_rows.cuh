@@ -68,18 +68,18 @@ __device__ __forceinline__ float2 load_once(const T* p) {
 // those loads long before it runs out of FMA slots (FP16, 65536 points, 2048
 // lines: 0.492 ms with it).
 //   f[0 .. 7): w^1 ... w^7;  f[7 .. 7 + A / 8 - 1): w^8, w^16, ...
-template <int A, class F>
+template <int A, bool FINE, class F>
 __device__ __forceinline__ void twiddled_column_dft(float2 (&z)[A], const float2 (&f)[6 + A / 8], const F& emit) {
   constexpr int R2 = A / 8;                      // radix of the last butterflies: 8 or 4
-  dft8_column<0, R2>(z);
-  dft8_column<1, R2>(z);
-  dft8_column<2, R2>(z);
-  dft8_column<3, R2>(z);
+  dft8_column<0, R2, FINE>(z);
+  dft8_column<1, R2, FINE>(z);
+  dft8_column<2, R2, FINE>(z);
+  dft8_column<3, R2, FINE>(z);
   if constexpr (R2 == 8) {
-    dft8_column<4, R2>(z);
-    dft8_column<5, R2>(z);
-    dft8_column<6, R2>(z);
-    dft8_column<7, R2>(z);
+    dft8_column<4, R2, FINE>(z);
+    dft8_column<5, R2, FINE>(z);
+    dft8_column<6, R2, FINE>(z);
+    dft8_column<7, R2, FINE>(z);
   }
 #pragma unroll
   for (int k2 = 0; k2 < 8; ++k2) {
@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(128, 3) fft_long_kernel(const RowArgs a) {
   using S = LongShape<N>;
   constexpr int A = S::A, C = S::C, P = S::P;
   constexpr float kInvN = 1.0f / float(N);
+  constexpr bool kFine = std::is_same<TS, float2>::value;   // see mul_root
   extern __shared__ float4 smem_long[];
   __shared__ __align__(8) uint64_t bar;
   chain_begin();
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(128, 3) fft_long_kernel(const RowArgs a) {
       slot[d] = mapa(base + uint32_t(n2) * kWord, d);
       rbar[d] = mapa(bar_local, d);
     }
-    twiddled_column_dft<A>(z, f, [&](int k1, float2 x) {
+    twiddled_column_dft<A, kFine>(z, f, [&](int k1, float2 x) {
       if constexpr (H16ROW) {
         st_async_b32(slot[k1 / 8] + uint32_t((k1 % 8) * 1024) * kWord, half2_bits(x), rbar[k1 / 8]);
       } else {
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(128, 3) fft_long_kernel(const RowArgs a) {
       cluster_barrier_relaxed();
       return;
     }
-    Dft<64>::run(v);
+    Dft<64, kFine>::run(v);
     float4* dst = reinterpret_cast<float4*>(sm + row * S::kRowPitch + t * 66);
 #pragma unroll
     for (int r = 0; r < P; r += 2) dst[r / 2] = make_float4(v[r].x, v[r].y, v[r + 1].x, v[r + 1].y);

@@ -75,7 +75,7 @@ struct WideNoHook {
   __device__ __forceinline__ void operator()() const {}
 };
 
-template <int N, int Ns, bool SPLIT>
+template <int N, int Ns, bool SPLIT, bool FINE>
 struct WidePass {
   static constexpr int P = WideShape<N>::P, T = WideShape<N>::T;
   static constexpr int R = wide_radix<N>(Ns);
@@ -105,8 +105,8 @@ struct WidePass {
   __device__ __forceinline__ static void run(float2 (&v)[P], const float4* __restrict__ tw, float* __restrict__ sm,
                                              int t, bool war, const H& after_last_read) {
     if constexpr (SPLIT && !kLast) {
-      static_assert(Ns == 1 && R == P && P % 4 == 0 && WidePass<N, R, SPLIT>::kLast, "split exchange: two passes");
-      Dft<R>::run(v);
+      static_assert(Ns == 1 && R == P && P % 4 == 0 && WidePass<N, R, SPLIT, FINE>::kLast, "split exchange: two passes");
+      Dft<R, FINE>::run(v);
       if (war) wide_sync<N>();
       constexpr int kPitch = P + 4;
       float4* dst = reinterpret_cast<float4*>(sm + t * kPitch);
@@ -122,9 +122,9 @@ struct WidePass {
       wide_sync<N>();
 #pragma unroll
       for (int m = 0; m < P; ++m) v[m] = make_float2(re[m], sm[t + (T * m / P) * kPitch + T * m % P]);
-      WidePass<N, R, SPLIT>::twiddle(v, tw, t);
+      WidePass<N, R, SPLIT, FINE>::twiddle(v, tw, t);
       after_last_read();
-      WidePass<N, R, SPLIT>::run(v, tw, sm, t, true, after_last_read);
+      WidePass<N, R, SPLIT, FINE>::run(v, tw, sm, t, true, after_last_read);
     } else {
       if constexpr (!kLast) {
         if (war) wide_sync<N>();
@@ -137,7 +137,7 @@ struct WidePass {
         float2 u[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) u[r] = v[b + B * r];
-        Dft<R>::run(u);
+        Dft<R, FINE>::run(u);
         if constexpr (kLast) {
 #pragma unroll
           for (int r = 0; r < R; ++r) o[b + B * r] = u[r];
@@ -155,7 +155,7 @@ struct WidePass {
 #pragma unroll
         for (int m = 0; m < P; ++m) v[m] = o[m];
       } else {
-        using Next = WidePass<N, Ns * R, SPLIT>;
+        using Next = WidePass<N, Ns * R, SPLIT, FINE>;
         wide_sync<N>();
 #pragma unroll
         for (int m = 0; m < P; ++m) v[m] = sm2[wide_pad<N>(t + T * m)];
@@ -167,11 +167,12 @@ struct WidePass {
   }
 };
 
-// Forward DFT of the line held in v (v[m] = x[t + T m] -> X[t + T m]).
-template <int N, bool SPLIT = false, class H = WideNoHook>
+// Forward DFT of the line held in v (v[m] = x[t + T m] -> X[t + T m]); FINE: see
+// mul_root.
+template <int N, bool SPLIT, bool FINE, class H = WideNoHook>
 __device__ __forceinline__ void wide_dft(float2 (&v)[WideShape<N>::P], const float4* __restrict__ tw,
                                          float* __restrict__ sm, int t, bool war, const H& after_last_read = H()) {
-  WidePass<N, 1, SPLIT>::run(v, tw, sm, t, war, after_last_read);
+  WidePass<N, 1, SPLIT, FINE>::run(v, tw, sm, t, war, after_last_read);
 }
 
 // v <- conj(v h) / N (Eq. 1's shift and conjugation behind the filter), h the
@@ -256,6 +257,7 @@ fft_wide_kernel(const RowArgs a) {
   using S = WideShape<N>;
   constexpr int P = S::P, T = S::T, G = S::G;
   constexpr bool kSplit = kWideSplit<N, MODE>;
+  constexpr bool kFine = std::is_same<TOut, float2>::value;
   static_assert(kWideOffered<N, TIn, MODE>, "see kWideOffered");
   extern __shared__ float4 smem_wide[];
   chain_begin();
@@ -295,18 +297,18 @@ fft_wide_kernel(const RowArgs a) {
       // longer lines' CTAs of 256 and 512 threads keep together and do not).
 #pragma unroll 1
       for (int it = 0; it < 2; ++it) {
-        wide_dft<N>(v, a.tw_wide, sm, t, it > 0);
+        wide_dft<N, false, kFine>(v, a.tw_wide, sm, t, it > 0);
         if (it == 0) wide_filter<N>(v, h);
       }
     } else {
-      wide_dft<N>(v, a.tw_wide, sm, t, false);
+      wide_dft<N, false, kFine>(v, a.tw_wide, sm, t, false);
       wide_filter<N>(v, h);
       int t2;   // opaque copy: the first transform's addresses are not kept live for the second
       asm volatile("mov.b32 %0, %1;" : "=r"(t2) : "r"(t));
-      wide_dft<N>(v, a.tw_wide, sm, t2, true);
+      wide_dft<N, false, kFine>(v, a.tw_wide, sm, t2, true);
     }
   } else {
-    wide_dft<N, kSplit>(v, a.tw_wide, sm, t, false);
+    wide_dft<N, kSplit, kFine>(v, a.tw_wide, sm, t, false);
   }
   wide_tail<N, MODE, SCALED>(v, a);
   if (active) {
@@ -329,6 +331,7 @@ __global__ void __launch_bounds__(WideShape<N>::kThreads, WideShape<N>::kMinBloc
 fft_wide_stream_kernel(const RowArgs a) {
   using S = WideShape<N>;
   constexpr int P = S::P, T = S::T;
+  constexpr bool kFine = std::is_same<TOut, float2>::value;
   static_assert(S::G == 1 && T > 32 && MODE != kCompress, "one line per CTA");
   static_assert(N * sizeof(TIn) <= wide_line_floats<N, false>() * sizeof(float), "the line fits the exchange buffer");
   extern __shared__ float4 smem_wide[];
@@ -364,7 +367,7 @@ fft_wide_stream_kernel(const RowArgs a) {
     }
     phase ^= 1;
     wide_head<N, MODE, SCALED>(v, a);
-    wide_dft<N>(v, a.tw_wide, sm, t, false, [&]() {
+    wide_dft<N, false, kFine>(v, a.tw_wide, sm, t, false, [&]() {
       __syncthreads();
       if (threadIdx.x == 0 && line + gridDim.x < a.lines) {
         fence_proxy_async_shared();
