@@ -1539,6 +1539,10 @@ int sar_make_filter(const void* ref, int64_t n, int peak_normalise, void* h_out,
   bfp::RowArgs a;
   int st = row_args(l, &a);
   if (st != BFPFFT_OK) return st;
+  // One line, on the 16-point kernel whatever its length: nothing is gained on
+  // another, and what is computed through the filter stays as it was.  The FP64
+  // entropy of an image follows every FP32 rounding of its filter (by 1e-8).
+  a.tw_wide = nullptr;
   a.in = ref;
   a.out = h_out;
   a.lines = 1;
