@@ -132,7 +132,9 @@ int bfpfft_plan_destroy(bfpfft_plan plan);
  * [16, 65536], mixed freely) at point offsets offset_pts[i] of the in / out
  * buffers.  By default batches of fewer than 2^23 points are all computed by
  * ONE persistent launch, larger ones by one launch per length
- * (BFPFFT_MANY_PER_LENGTH).  For the persistent launch the plan sorts
+ * (BFPFFT_MANY_PER_LENGTH) where that is faster: with few lengths from 2^23
+ * points on, with many from about 2 million points a length on.  For the
+ * persistent launch the plan sorts
  * the lines into tasks of 65,536 points of one length, largest length first;
  * thread-block clusters of 16 CTAs take every clusters-th task in turn (a
  * line of 65536 spans the whole cluster, shorter lines one CTA or part of

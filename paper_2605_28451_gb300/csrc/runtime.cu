@@ -505,8 +505,8 @@ struct bfpfft_plan_s {
                                         // persistent kernel's four-step lines (0)
   int fs_h16 = 0;                       // FP16 storage: four-step lines exchange their rows as FP16 words (1)
   int per_length = -1;                  // one dense-row launch per length over its listed lines (1), the persistent
-                                        // kernel (0), or by the batch's size (-1, see large_batch)
-  bool large_batch = false;             // at least kPerLengthPoints points
+                                        // kernel (0), or by the batch's lengths (-1, see prefers_per_length)
+  bool by_length = false;               // what prefers_per_length says
   std::mutex fork_mutex;                // the forks below serve one exec at a time
   int has_fourstep = 0;                 // some line has 8192 points or more
   long long len_first[kMaxLog2 + 1] = {};   // lines of 2^l points: first index into d_line_off ...
@@ -533,13 +533,34 @@ struct bfpfft_plan_s {
 
 namespace {
 
-// Uneven batches from this many points on run as one launch per length unless
-// told otherwise: the dense kernels of each length beat the persistent one,
-// whose CTAs are sized for every length at once, as soon as a length fills the
-// GPU (lengths 256 ... 65536, FP16, us per batch, persistent / per length: 2.2 M
-// points 23 / 31, 7.1 M 51 / 43, 25.7 M 166 / 106, 252 M 1545 / 780; lengths
-// 16 ... 1024: 2.8 M 20 / 29, 6.9 M 30 / 34).
+// Which schedule an untuned uneven batch takes: one launch per length, or the
+// persistent kernel.  The dense kernels of each length beat the persistent one,
+// whose CTAs are sized for every length at once, by the figures below for each
+// point (tenths of a picosecond; measured from 2^25 points of one length, FP16
+// and FP8 storage; FP32 saves more, of which a tenth more is counted).  Every
+// length after the first costs a launch, some 4 us of host time and ramp.  Lines
+// of 32768 points and more save 3.2 ps and count as 7, in every storage: their
+// launches overlap the shorter lengths' on another stream.  Below 2^23 points a
+// batch stays on the persistent kernel.  Times (persistent / per length, us a
+// batch, FP16): 13 lengths with equal shares of 8.4 M points 47 / 70, of 33.6 M
+// 164 / 142; nine (16 ... 4096) with 8.4 M 39 / 58, with 16.8 M 74 / 79, with
+// 33.6 M 140 / 127; three (256, 512, 1024) with 8.4 M 29 / 20; the ragged batch of
+// lengths 256 ... 65536, mostly in the longest, with 25.7 M 166 / 106 and 252 M
+// 1545 / 774.
 constexpr int64_t kPerLengthPoints = int64_t(1) << 23;
+constexpr double kPerLengthLaunchUs = 4.0;
+bool prefers_per_length(const int64_t (&points)[kMaxLog2 + 1], bool f32) {
+  int64_t total = 0;
+  int lengths = 0;
+  double saved = 0.0;
+  for (int l = kMinLog2; l <= kMaxLog2; ++l) {
+    const int tenths_ps = l <= 5 ? 18 : l <= 8 ? 12 : l <= 12 ? 15 : l <= 14 ? 30 : 70;
+    total += points[l];
+    lengths += points[l] > 0;
+    saved += double(points[l]) * tenths_ps * (f32 && l <= 14 ? 1.1e-7 : 1e-7);   // us
+  }
+  return total >= kPerLengthPoints && saved > kPerLengthLaunchUs * (lengths - 1);
+}
 
 void destroy_fork(Fork* f) {
   if (f->side) cudaStreamDestroy(f->side);
@@ -737,10 +758,10 @@ static int exec_per_length(bfpfft_plan plan, const void* in, void* out, cudaStre
 }
 
 static int exec_many(bfpfft_plan plan, const void* in, void* out, cudaStream_t s) {
-  // An untuned plan goes by its size, unless BFPFFT_ROWS names a form of the
+  // An untuned plan goes by its lengths, unless BFPFFT_ROWS names a form of the
   // persistent kernel.
-  const bool by_size = plan->per_length < 0 && plan->large_batch && std::getenv("BFPFFT_ROWS") == nullptr;
-  if (plan->per_length > 0 || by_size) return exec_per_length(plan, in, out, s);
+  const bool by_length = plan->per_length < 0 && plan->by_length && std::getenv("BFPFFT_ROWS") == nullptr;
+  if (plan->per_length > 0 || by_length) return exec_per_length(plan, in, out, s);
   bfp::UnevenArgs a{};
   a.in = in;
   a.out = out;
@@ -1152,9 +1173,9 @@ int bfpfft_plan_create_many(bfpfft_plan* out, int64_t count, const int64_t* n, c
   p->many = true;
   p->kind = kind;
   p->num_tasks = int(tasks.size());
-  int64_t points = 0;
-  for (int64_t i = 0; i < count; ++i) points += n[i];
-  p->large_batch = points >= kPerLengthPoints;
+  int64_t points[kMaxLog2 + 1] = {};
+  for (int l = kMinLog2; l <= kMaxLog2; ++l) points[l] = int64_t(by_class[l].size()) << l;
+  p->by_length = prefers_per_length(points, dtype == BFPFFT_F32);
   // Tasks are sorted longest first: lines of 65536 and 32768 points come first.
   p->first_short_task = 0;
   for (const auto& t : tasks) {
