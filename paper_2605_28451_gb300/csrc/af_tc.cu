@@ -59,7 +59,8 @@ __device__ __forceinline__ float2 load_point<float2>(const float2* p) {
 }
 
 // The last pass of a transform, with the accumulators handed to `epi(h, rho,
-// d)` for both M tiles (rows rho = tau and 128 + tau).
+// d)` for both M tiles (rows rho = tau and 128 + tau), unless this thread's wait
+// expired.
 template <class Epi>
 __device__ __forceinline__ bool tc_last_pass(int* status, uint64_t* bar, uint32_t tmem, uint32_t lane_tmem,
                                              uint32_t a_base, uint32_t b, uint32_t& phase, Epi epi) {
@@ -68,7 +69,7 @@ __device__ __forceinline__ bool tc_last_pass(int* status, uint64_t* bar, uint32_
   for (int h = 0; h < 2; ++h) {
     uint32_t d[32];
     tc::ld32(lane_tmem + uint32_t(32 * h), d);
-    epi(h, int(threadIdx.x) + 128 * h, d);
+    if (tc_valid(phase)) epi(h, int(threadIdx.x) + 128 * h, d);
   }
   tc::fence_before();
   return true;

@@ -182,9 +182,10 @@ __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::aft
 // and overwrite A at once: its own wait has seen the commit, so no second
 // barrier follows.  A wait that expires is kept in bit 31 of `phase`; the next
 // barrier makes it known to all threads, and the call returns false to all of
-// them (until then the thread works on with values that are not valid, as the
-// recorded timeout says).
+// them.  Until then the thread works on with values that are not valid; they go
+// no further than the A tile: what leaves the chip asks for tc_valid first.
 constexpr uint32_t kTcExpired = 0x80000000u;
+__device__ __forceinline__ bool tc_valid(uint32_t phase) { return (phase & kTcExpired) == 0u; }
 
 struct TcNothing {
   __device__ __forceinline__ void operator()() const {}
@@ -308,7 +309,7 @@ __device__ __forceinline__ bool tc_pass(const RowArgs& a, long long line, unsign
       }
     } else if constexpr (FILTER) {
       tc_filter_to_a<false>(sA, rho, d, a.h + line * a.h_stride + rho);
-    } else {
+    } else if (tc_valid(phase)) {
       // The inverse's final conjugation is folded into the last pass's matrix.
       TOut* out = static_cast<TOut*>(a.out) + line * a.out_stride + rho;
 #pragma unroll
