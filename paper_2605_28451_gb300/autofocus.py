@@ -17,6 +17,7 @@ Only argument marshalling happens here.
 from __future__ import annotations
 
 import torch
+from torch.autograd import forward_ad
 
 from . import bfpfft as B
 
@@ -38,12 +39,13 @@ class Workspace:
 KEEP_BYTES = 512 << 20   # largest state kept between forward and backward
 
 
-def _versions(*tensors):
+def _versions(rc, ha):
     """The tensors' version counters, or None where one has none to tell a change
     by (made under inference_mode, or not torch's)."""
-    if any(not isinstance(x, torch.Tensor) or x.is_inference() for x in tensors):
-        return None
-    return tuple(x._version for x in tensors)
+    for x in (rc, ha):
+        if not isinstance(x, torch.Tensor) or x.is_inference():
+            return None
+    return rc._version, ha._version
 
 
 def _saved_tensor_hooks() -> bool:
@@ -52,6 +54,19 @@ def _saved_tensor_hooks() -> bool:
     in a fraction of the time that moving it takes, is not handed to them."""
     top = getattr(torch._C._autograd, "_top_saved_tensors_default_hooks", None)
     return top is not None and top(False) is not None
+
+
+def _address(g):
+    """The address of an upstream gradient if the value there is all there is to it,
+    else None: it carries a graph or a tangent on, waits for a negation, or is a
+    wrapper (a batch) without an address."""
+    if torch.is_grad_enabled() or getattr(forward_ad, "_current_level", 0) >= 0 or type(g) is not torch.Tensor \
+            or g.is_neg():
+        return None
+    try:
+        return g.data_ptr()
+    except RuntimeError:
+        return None
 
 
 class SarEntropy(torch.autograd.Function):
@@ -79,8 +94,9 @@ class SarEntropy(torch.autograd.Function):
                     state = None
                 if state is not None:
                     e = torch.empty((), dtype=torch.float64, device=phi_c.device)
-                    B.sar_autofocus_entropy_keep(rc, rc_dtype, phi_c, ha, n_az, n_rg, ws.stats, e, state, size,
-                                                 ws.buf, ws.bytes)
+                    # Addresses of what nobody else holds: no version counters to advance.
+                    B.sar_autofocus_entropy_keep(rc, rc_dtype, phi_c, ha, n_az, n_rg, ws.stats, e.data_ptr(),
+                                                 state.data_ptr(), size, ws.buf, ws.bytes)
                     ctx.save_for_backward(phi_c, state)
                     ctx.versions = versions
                     return e
@@ -94,17 +110,20 @@ class SarEntropy(torch.autograd.Function):
         rc, ha, ws = ctx.rc, ctx.ha, ctx.ws
         n_rg, n_az = rc.shape[0], rc.shape[1]
         grad = torch.empty(n_az, dtype=torch.float32, device=phi_c.device)
+        scale = None
         if kept and ws.arith == B.ARITH_F32 and ctx.versions == _versions(rc, ha):
             state = kept[0]
-            B.sar_autofocus_grad_kept(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, state, state.numel(), None, grad,
-                                      ws.stats, ws.buf, ws.bytes)
+            # The library multiplies by g_e where that loses nothing: a product in
+            # torch takes another 10 us of host time.
+            scale = _address(g_e)
+            B.sar_autofocus_grad_kept(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, state, state.numel(), scale,
+                                      grad.data_ptr(), ws.stats, ws.buf, ws.bytes)
         else:
-            B.sar_autofocus_grad(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, grad, ws.stats, ws.buf, ws.bytes,
+            B.sar_autofocus_grad(rc, ctx.rc_dtype, phi_c, ha, n_az, n_rg, grad.data_ptr(), ws.stats, ws.buf, ws.bytes,
                                  arith=ws.arith)
-        # A torch product, not the library's scale argument: g_e may carry a graph
-        # (create_graph), a batch (is_grads_batched) or a tangent (forward mode),
-        # which a raw pointer would lose.  g_e is a scalar: the product is FP32.
-        return g_e * grad, None, None, None, None, None
+        if scale is None:
+            grad = g_e * grad            # g_e is a scalar: the product is FP32
+        return grad, None, None, None, None, None
 
 
 def entropy(phi, rc, ha, rc_dtype: int, ws: Workspace):

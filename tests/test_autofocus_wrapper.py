@@ -16,6 +16,13 @@ def column_sums(rc):
     return rc.sum(0)
 
 
+def floats(address, count, ctype=ctypes.c_float):
+    """The numbers at an address the wrapper handed over (the library never sees the tensors themselves)."""
+    address = address if isinstance(address, int) else address.data_ptr()
+    return torch.frombuffer((ctype * count).from_address(address), dtype=torch.float32 if ctype is ctypes.c_float
+                            else torch.float64)
+
+
 class Library:
     """The calls SarEntropy makes, and which of them were made."""
 
@@ -32,19 +39,19 @@ class Library:
 
     def entropy_keep(self, rc, rc_dtype, phi, ha, n_az, n_rg, stats, e, state, state_bytes, ws, ws_bytes, stream=None):
         self.calls.append("entropy_keep")
-        e.copy_((column_sums(rc) * phi).sum())
-        state[:4 * n_az].view(torch.float32).copy_(column_sums(rc))
+        floats(e, 1, ctypes.c_double).copy_((column_sums(rc) * phi).sum())
+        floats(state, n_az).copy_(column_sums(rc))
 
     def grad(self, rc, rc_dtype, phi, ha, n_az, n_rg, grad, stats, ws, ws_bytes, arith=B.ARITH_F32, stream=None):
         self.calls.append("grad")
-        grad.copy_(column_sums(rc))
+        floats(grad, n_az).copy_(column_sums(rc))
 
     def grad_kept(self, rc, rc_dtype, phi, ha, n_az, n_rg, state, state_bytes, scale, grad, stats, ws, ws_bytes,
                   stream=None):
         self.calls.append("grad_kept")
-        grad.copy_(state[:4 * n_az].view(torch.float32))
-        if scale is not None:   # the library reads it through its address
-            grad.mul_(ctypes.c_double.from_address(scale.data_ptr()).value)
+        floats(grad, n_az).copy_(floats(state, n_az))
+        if scale is not None:
+            floats(grad, n_az).mul_(floats(scale, 1, ctypes.c_double).item())
 
 
 @pytest.fixture
@@ -93,6 +100,22 @@ def test_tangent_of_the_upstream_gradient(library):
         grad, = torch.autograd.grad(e, phi, grad_outputs=up)
         primal, tangent = torch.autograd.forward_ad.unpack_dual(grad)
     assert torch.equal(primal, 2.0 * column_sums(rc)) and torch.equal(tangent, 7.0 * column_sums(rc))
+
+
+@pytest.mark.parametrize("factor", [1.0, -2.5])
+def test_plain_upstream_gradient(library, factor):
+    rc, ha, phi, ws = scene(8)
+    grad, = torch.autograd.grad(GA.entropy(phi, rc, ha, B.F32, ws) * factor, phi)
+    assert grad.dtype == torch.float32 and torch.equal(grad, factor * column_sums(rc))
+
+
+def test_upstream_gradient_with_a_pending_negation(library):
+    """The imaginary part of a lazily conjugated gradient: its sign is a flag, not in memory."""
+    rc, ha, phi, ws = scene(9)
+    z = torch.complex(torch.zeros((), dtype=torch.float64), GA.entropy(phi, rc, ha, B.F32, ws))
+    loss = (z.conj() * torch.tensor(1 + 2j, dtype=torch.complex128)).real          # 2 E
+    grad, = torch.autograd.grad(loss, phi)
+    assert torch.equal(grad, 2.0 * column_sums(rc))
 
 
 @pytest.mark.parametrize("which", ["rc", "ha"])
