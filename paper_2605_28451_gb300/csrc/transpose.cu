@@ -15,6 +15,12 @@ namespace bfp {
 
 namespace {
 
+// One 16-byte vector of elements, read and written whole.
+template <class T>
+struct alignas(16) TileVec {
+  T v[16 / sizeof(T)];
+};
+
 // Tiles of TILE x TILE elements, TILE * sizeof(T) = 256 bytes: 64 x 64 half2
 // or 32 x 32 float2.  256 threads, 16 x 16: each takes a block of VEC x VEC
 // elements, VEC rows of one 16-byte vector, turns it by the naming of its
@@ -47,7 +53,7 @@ struct TileIo {
     c0 = (long long)(b % col_tiles) * TILE;
   }
   // This thread's block of tile b: rows VEC rb ... of columns VEC cb ....
-  __device__ void load(const T* in, unsigned b, int cb, int rb, T (&e)[VEC][VEC]) const {
+  __device__ void load(const T* in, unsigned b, int cb, int rb, TileVec<T> (&e)[VEC]) const {
     long long r0, c0;
     origin(b, r0, c0);
     const bool vec = r0 + TILE <= rows && c0 + TILE <= cols && cols % VEC == 0;
@@ -55,11 +61,11 @@ struct TileIo {
 #pragma unroll
     for (int k = 0; k < VEC; ++k) {
       if (vec) {
-        *reinterpret_cast<uint4*>(e[k]) = __ldcs(reinterpret_cast<const uint4*>(in + (r + k) * cols + c));
+        *reinterpret_cast<uint4*>(&e[k]) = __ldcs(reinterpret_cast<const uint4*>(in + (r + k) * cols + c));
       } else {
 #pragma unroll
         for (int i = 0; i < VEC; ++i) {
-          if (r + k < rows && c + i < cols) e[k][i] = in[(r + k) * cols + c + i];
+          if (r + k < rows && c + i < cols) e[k].v[i] = in[(r + k) * cols + c + i];
         }
       }
     }
@@ -77,15 +83,15 @@ __global__ void __launch_bounds__(256, 5) transpose_kernel(const T* in, T* out, 
   const int lane16 = threadIdx.x % 16, row16 = threadIdx.x / 16;
   unsigned b = blockIdx.x;
   if (b >= tiles) return;
-  T e[VEC][VEC];
+  TileVec<T> e[VEC];
   io.load(in, b, lane16, row16, e);
   for (; b < tiles; b += gridDim.x) {
 #pragma unroll
     for (int i = 0; i < VEC; ++i) {
-      T w[VEC];
+      TileVec<T> w;
 #pragma unroll
-      for (int k = 0; k < VEC; ++k) w[k] = e[k][i];
-      tile[16 * (lane16 * VEC + i) + (row16 ^ (lane16 & 7))] = *reinterpret_cast<const uint4*>(w);
+      for (int k = 0; k < VEC; ++k) w.v[k] = e[k].v[i];
+      tile[16 * (lane16 * VEC + i) + (row16 ^ (lane16 & 7))] = *reinterpret_cast<const uint4*>(&w);
     }
     __syncthreads();
     if (b + gridDim.x < tiles) io.load(in, b + gridDim.x, lane16, row16, e);   // in flight while this tile is written
