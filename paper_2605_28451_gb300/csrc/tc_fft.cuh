@@ -230,10 +230,11 @@ __device__ __forceinline__ void tc_store_row0(unsigned char* sA, int j, const ui
 
 // The last pass of a forward transform whose spectrum is filtered: output q
 // of butterfly rho is bin k = rho + 256 q; conj(X[k] H[k]) / N (H conjugated
-// first when CONJ_H) rounded to FP16 is the inverse's pass-0 input.
+// first when CONJ_H) rounded to FP16 is the inverse's pass-0 input.  No
+// __restrict__ on hk: an earlier kernel may have written it (see chain_begin).
 template <bool CONJ_H>
 __device__ __forceinline__ void tc_filter_to_a(unsigned char* sA, int rho, const uint32_t (&d)[32],
-                                               const float2* __restrict__ hk) {
+                                               const float2* hk) {
   const float inv_n = 1.0f / float(tc::kN);
   uint32_t x[16];
 #pragma unroll

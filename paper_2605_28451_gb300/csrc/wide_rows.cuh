@@ -179,9 +179,10 @@ __device__ __forceinline__ void wide_dft(float2 (&v)[WideShape<N>::P], const flo
 // thread's first filter point.  Loads go in groups of eight, for the short
 // lines one group ahead of the products; more in flight do not fit beside the
 // line's registers (nor does the second group at 8192 points and more, 3 %
-// slower with it).
+// slower with it).  No __restrict__: an earlier kernel may have written h (see
+// chain_begin).
 template <int N>
-__device__ __forceinline__ void wide_filter(float2 (&v)[WideShape<N>::P], const float2* __restrict__ h) {
+__device__ __forceinline__ void wide_filter(float2 (&v)[WideShape<N>::P], const float2* h) {
   constexpr int P = WideShape<N>::P, T = WideShape<N>::T;
   constexpr float kInvN = 1.0f / float(N);
   constexpr int kAhead = N <= 4096 ? 8 : 0;
