@@ -779,6 +779,19 @@ struct LaunchSetup {
   int resident;
 };
 
+// SMs of the device, once per process (as the kernels' set-ups); 1 if it cannot
+// be asked.
+inline int sm_count() {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      n = 0;
+    return n > 0 ? n : 1;
+  }();
+  return sms;
+}
+
 template <class K>
 LaunchSetup setup_kernel(K kern, int threads, size_t smem) {
   LaunchSetup r{cudaSuccess, 0};
@@ -1306,7 +1319,7 @@ cudaError_t launch_rows_n(const RowArgs& a, cudaStream_t stream) {
   if constexpr (!TLOAD && !TSTORE && !NAIVE && N >= 512) {
     if constexpr (kWideOffered<N, TIn, MODE>) {
       if ((a.variant == kRowsPlain4L2 || a.variant == kRowsPlain4) && a.tw_wide != nullptr &&
-          a.lines >= kWideMinLines<N>)
+          a.lines >= (long long)kWideLinesPerSm<N> * sm_count())
         return launch_wide_n<N, TIn, TOut, MODE, SCALED>(a, stream, a.variant == kRowsPlain4L2);
     }
   }

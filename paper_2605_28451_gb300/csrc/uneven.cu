@@ -189,7 +189,7 @@ cudaError_t launch_typed(const UnevenArgs& a, int clusters, cudaStream_t s) {
   // Chained only up to a CTA per SM: 20 transforms (1.4e5 points) 10.3 -> 7.75
   // us; with the GPU full the clusters no longer start together, and 100 (1.1e6
   // points) take 17.9 instead of 16.5, 400 38.3 instead of 35.3.
-  const bool chained = clusters * kClusterCtas <= 152;
+  const bool chained = clusters * kClusterCtas <= sm_count();
   return launch_chained(kern, clusters * kClusterCtas, kCta, uneven_smem_bytes<TS>(), kClusterCtas, chained, s, a);
 }
 

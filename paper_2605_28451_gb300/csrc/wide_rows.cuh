@@ -250,7 +250,7 @@ constexpr bool kWideSplit = N == 4096 && MODE == kForward;
 template <int N, class TIn, int MODE>
 constexpr bool kWideOffered = WideShape<N>::P == 32 || (MODE != kCompress && !std::is_same<TIn, float2>::value);
 template <int N>
-constexpr long long kWideMinLines = N == 2048 ? 1216 : N == 4096 ? 1824 : 0;   // 8 and 12 lines per SM
+constexpr int kWideLinesPerSm = N == 2048 ? 8 : N == 4096 ? 12 : 0;   // at least: 1216 and 1824 lines on 152 SMs
 
 template <int N, class TIn, class TOut, int MODE, bool SCALED>
 __global__ void __launch_bounds__(WideShape<N>::kThreads, WideShape<N>::kMinBlocks)
