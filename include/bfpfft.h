@@ -238,6 +238,17 @@ int bfpfft_plan_scale_exp(bfpfft_plan plan, int* in_exp, int* out_exp);
 int bfpfft_device_status(int* status);
 
 /*
+ * Give the scratch memory that no call is using back to the driver, after a
+ * device-wide synchronisation.  The SAR, autofocus and two-pass calls take
+ * their scratch from a pool of the library's, one per device, which keeps what
+ * it has for the next call: the largest amount that calls of all streams had
+ * in use at once (a call's own amount is stated with it).  Applies to the
+ * current device; the next call takes memory from the driver again.  Not inside
+ * a stream capture.  Errors: CUDA.
+ */
+int bfpfft_release_scratch(void);
+
+/*
  * Read and clear the plan's own status word after a device-wide
  * synchronisation (call it on the plan's device).  Its kernels record there:
  *   BFPFFT_ERR_TIMEOUT   a bounded device-side wait expired (bulk-copy
@@ -492,10 +503,11 @@ int sar_rda_image(const void* raw, int raw_dtype, void* img, int img_dtype, cons
  *   S = sum q,  E = -sum (q/S) ln(q/S) = ln S - (1/S) sum q ln q,
  *   dE/dphi[n] = 2 sum_r Im( conj((A^H G)[r][n]) v[r][n] ),
  *   G = -(ln(q/S) + E) / S . I,  A^H = IDFT(DFT(.) . conj(Ha)).
- * A gradient call keeps the image (FP32) between its two passes in scratch from
- * the library's stream-ordered pool, up to 512 MiB; where it does not fit, and
- * inside a stream capture, the gradient pass computes the forward transforms
- * again.  FP32 arithmetic; FP64 sums across CTAs.
+ * A gradient call keeps the image (FP32, n_az * n_rg * 8 bytes) between its two
+ * passes in scratch from the library's stream-ordered pool, up to 512 MiB (the
+ * pool keeps the memory afterwards: bfpfft_release_scratch); where it does not
+ * fit, and inside a stream capture, the gradient pass computes the forward
+ * transforms again.  FP32 arithmetic; FP64 sums across CTAs.
  * Layout: rc is [n_rg][n_az] (each row one range bin's azimuth line, as written
  * by sar_range_compress with transpose_out = 1), dtype BFPFFT_F32 or
  * BFPFFT_F16_BFP; phi float[n_az], Ha float2[n_az] (device).

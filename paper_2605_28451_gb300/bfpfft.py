@@ -68,6 +68,7 @@ SIGNATURES = {
     "bfpfft_plan_destroy": (ctypes.c_int, [_vp]),
     "bfpfft_plan_scale_exp": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]),
     "bfpfft_device_status": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int)]),
+    "bfpfft_release_scratch": (ctypes.c_int, []),
     "bfpfft_plan_status": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int)]),
     "bfpfft_plan_set_flags": (ctypes.c_int, [_vp, ctypes.c_int]),
     "bfpfft_plan_set_many_schedule": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int]),
@@ -294,6 +295,11 @@ def bfpfft_device_status() -> int:
     st = ctypes.c_int()
     _check(lib().bfpfft_device_status(ctypes.byref(st)), "bfpfft_device_status")
     return st.value
+
+
+def bfpfft_release_scratch():
+    """Synchronise the device, then give its unused scratch memory back to the driver."""
+    _check(lib().bfpfft_release_scratch(), "bfpfft_release_scratch")
 
 
 def bfpfft_plan_status(plan: Plan) -> int:

@@ -314,19 +314,20 @@ bool sar_split_turns() {
 
 // Stream-ordered scratch from a library-owned pool per device that keeps its
 // memory between calls (release threshold: never), so repeated calls neither
-// synchronise nor return memory to the driver.
+// synchronise nor return memory to the driver; bfpfft_release_scratch does.
+std::mutex g_pool_mutex;
+std::map<int, cudaMemPool_t> g_pools;
+
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
-  static std::mutex mu;
-  static std::map<int, cudaMemPool_t> pools;
   if (fault("alloc")) return cudaErrorMemoryAllocation;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   cudaMemPool_t pool;
   {
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = pools.find(dev);
-    if (it == pools.end()) {
+    std::lock_guard<std::mutex> lock(g_pool_mutex);
+    auto it = g_pools.find(dev);
+    if (it == g_pools.end()) {
       cudaMemPoolProps props = {};
       props.allocType = cudaMemAllocationTypePinned;
       props.location.type = cudaMemLocationTypeDevice;
@@ -334,7 +335,7 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
       if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
       uint64_t keep = UINT64_MAX;
       if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
-      pools[dev] = pool;
+      g_pools[dev] = pool;
     } else {
       pool = it->second;
     }
@@ -1385,6 +1386,17 @@ int bfpfft_device_status(int* status) {
   return cuda_status(e);
 }
 
+int bfpfft_release_scratch(void) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_status(e);
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  auto it = g_pools.find(dev);
+  if (it == g_pools.end()) return BFPFFT_OK;
+  if ((e = cudaDeviceSynchronize()) == cudaSuccess) e = cudaMemPoolTrimTo(it->second, 0);
+  return cuda_status(e);
+}
+
 int bfpfft_plan_status(bfpfft_plan plan, int* status) {
   if (plan == nullptr || status == nullptr) return BFPFFT_ERR_INVALID_ARG;
   cudaError_t e = cudaDeviceSynchronize();
@@ -1829,7 +1841,8 @@ size_t sar_autofocus_workspace_bytes(int64_t n_az) {
 }
 
 // A gradient keeps the FP32 image of its entropy pass in stream-ordered scratch
-// up to this size (16383 range bins of 4096 pulses); beyond it, without memory
+// (which stays with the pool, see scratch_alloc) up to this size (16383 range
+// bins of 4096 pulses); beyond it, without memory
 // for it, or inside a stream capture, the gradient pass computes it again.
 // Kept, a gradient step on 4096 x 4096 FP16 data takes 229 us, computed again
 // 289.
