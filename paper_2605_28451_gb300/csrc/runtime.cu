@@ -349,8 +349,7 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
 // into L2 the lines of the CTA one resident wave later -- the fastest
 // exact-numerics variant measured on GB300; unknown names: the pipelined
 // kernel.
-int rows_variant() {
-  const char* v = std::getenv("BFPFFT_ROWS");
+int rows_variant(const char* v) {
   if (v == nullptr) return bfp::kRowsPlain4L2;
   static const struct { const char* name; int code; } kNames[] = {
       {"tma", bfp::kRowsTma},         {"plain", bfp::kRowsPlain},    {"pp", bfp::kRowsPlainPP},
@@ -363,6 +362,7 @@ int rows_variant() {
     if (std::strcmp(v, k.name) == 0) return k.code;
   return bfp::kRowsTma;
 }
+int rows_variant() { return rows_variant(std::getenv("BFPFFT_ROWS")); }
 
 // The 16-point DFT matrix of the tensor-core variant in real form, FP16,
 // [n][k]: B[2q][2r] = Re W, B[2q][2r+1] = -Im W, B[2q+1][2r] = Im W,
@@ -1266,7 +1266,8 @@ int bfpfft_exec(bfpfft_plan plan, const void* in, void* out, void* stream) {
   a.h = nullptr;
   a.status = plan->status;
   a.finite_flag = (plan->flags & BFPFFT_CHECK_FINITE) ? plan->status : nullptr;
-  a.variant = std::getenv("BFPFFT_ROWS") == nullptr && plan->variant >= 0 ? plan->variant : rows_variant();
+  const char* rows = std::getenv("BFPFFT_ROWS");
+  a.variant = rows == nullptr && plan->variant >= 0 ? plan->variant : rows_variant(rows);
   if (!device_memory(in)) {
     a.variant = without_l2(a.variant);
     a.no_prefetch = 1;
