@@ -719,10 +719,12 @@ def _bench_autofocus(B, torch, dev, stream):
             e1.synchronize()
             ts.append(e0.elapsed_time(e1))
         t = statistics.median(ts)
-        # entropy pass: 2 transforms per range bin; gradient pass: 4 (recomputed forward + adjoint)
-        flops = 6 * n * 5 * n * 12
+        # entropy pass: 2 transforms per range bin; gradient pass: 2 from the kept image (FP32 arithmetic), 4
+        # where the image is computed again (tensor cores).  rc is read once by each, and once more with the latter.
+        transforms, reads = (4, 2) if arith == B.ARITH_F32 else (6, 3)
+        flops = transforms * n * 5 * n * 12
         out[name] = {"ms_median_l2_flushed": round(t, 4), "gflops": round(flops / (t * 1e-3) / 1e9, 1),
-                     "alg_gbs": round(3 * 4 * n * n / (t * 1e-3) / 1e9, 1)}
+                     "alg_gbs": round(reads * 4 * n * n / (t * 1e-3) / 1e9, 1)}
         g = grad.double()
         if ref_grad is None:
             ref_grad = g.clone()

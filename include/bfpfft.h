@@ -108,6 +108,11 @@ const char* bfpfft_error_string(int status);
  * FP8 plans carry static block exponents, see bfpfft_plan_scale_exp().
  * batch may be 0 (exec is then a no-op).  The plan allocates its twiddle
  * table on the current device; it must be executed on that device.
+ * The number of lines has a say in which kernel runs (2048 and 4096 points from
+ * 8 and 12 lines per SM on; 32768 and 65536 from 655,360 points on; an uneven
+ * batch by its lengths), and the kernels round differently in FP32: a line's
+ * bits repeat from call to call of one plan, but may differ in their last
+ * places between plans of different batches.
  * Errors: INVALID_ARG (out NULL, batch < 0, unknown dtype or direction),
  * UNSUPPORTED (n not a power of two in [16, 65536]), OOM, CUDA.
  * On error *out is set to NULL.

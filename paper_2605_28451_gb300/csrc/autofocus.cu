@@ -22,11 +22,11 @@
 //   af_kernel<kAfRecompute> the same without scratch: I[r] is computed again
 //   af_grad_kernel          sum of the partial gradients in FP64 (32 slices per 32 pulses)
 //
-// Arithmetic bounds the passes (FMA pipe 50 to 60 % busy), so a gradient step
-// costs its transforms: four with I kept, six when it is computed again.  Kept,
-// I moves 16 bytes a pixel more through L2 and HBM, which the arithmetic
-// covers.  Measured on GB300, 4096 x 4096 FP16 rc, one gradient step: see
-// kAfKeepBytes.
+// A gradient step costs its transforms: four with I kept, six when it is computed
+// again.  Neither pass fills a pipe (entropy and adjoint: issue slots 52 and 53 %
+// busy, FMA 44 %, L1 52 and 46 %, at two CTAs of 256 threads per SM).  Keeping I
+// costs the entropy pass 11 us of stores and saves the adjoint 77 us (104 instead
+// of 181; 4096 x 4096, FP16 rc, GB300).  The whole step: see kAfKeepBytes.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -126,10 +126,9 @@ enum AfPass : int { kAfEntropy = 0, kAfAdjoint = 1, kAfRecompute = 2 };
 
 // Resident CTAs per SM: two of 256 threads at 128 registers, one of 512.  More
 // do not help: the entropy pass takes 98 to 102 us a call at two, three or four
-// (its logarithms and transforms keep the issue slots 57 % busy), the adjoint
-// pass is slower at four (a step takes 249 us against 224) and leaves more
-// partial gradients to sum.  The number also fixes which rows a CTA's FP32
-// partial of the entropy adds up.
+// (issue slots 52 % busy at two), the adjoint pass is slower at four (a step
+// takes 249 us against 224) and leaves more partial gradients to sum.  The
+// number also fixes which rows a CTA's FP32 partial of the entropy adds up.
 template <int N, int PASS>
 constexpr int af_min_blocks() {
   return RowShape<N>::kThreads >= 512 ? 1 : 2;

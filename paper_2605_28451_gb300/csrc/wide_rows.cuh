@@ -7,7 +7,7 @@
 // instructions per thread for every point a thread moves through them; it is
 // bound by those two pipes (78 % and 61 % busy) at 63 % of the HBM copy rate.
 // With 64 points per thread the line is 64 x 64: one exchange, one set of
-// twiddles, 8 wavefronts and 35 instructions a point.  Passes (N = P * ...):
+// twiddles, 8 wavefronts and 39 instructions a point.  Passes (N = P * ...):
 //   512 = 32 x 16, 1024 = 32 x 32 (32 points per thread; a line is a half or a
 //   whole warp, so the exchange needs no CTA barrier), 2048 = 64 x 32 (one
 //   warp), 4096 = 64 x 64 (two warps), 8192 = 32 x 16 x 16 and 16384 =
