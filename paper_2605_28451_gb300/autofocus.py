@@ -42,18 +42,16 @@ KEEP_BYTES = 512 << 20   # largest state kept between forward and backward
 def _versions(rc, ha):
     """The tensors' version counters, or None where one has none to tell a change
     by (made under inference_mode, or not torch's)."""
-    for x in (rc, ha):
-        if not isinstance(x, torch.Tensor) or x.is_inference():
-            return None
-    return rc._version, ha._version
+    try:
+        return rc._version, ha._version
+    except (RuntimeError, AttributeError):
+        return None
 
 
-def _saved_tensor_hooks() -> bool:
-    """Whether saved tensors pass through hooks (offloading, compression,
-    checkpointing).  Those are meant for saved inputs: the image, computed again
-    in a fraction of the time that moving it takes, is not handed to them."""
-    top = getattr(torch._C._autograd, "_top_saved_tensors_default_hooks", None)
-    return top is not None and top(False) is not None
+# The saved-tensor hooks in force, if any (offloading, compression,
+# checkpointing).  Those are meant for saved inputs: the image, computed again in
+# a fraction of the time that moving it takes, is not handed to them.
+_saved_tensor_hooks = getattr(torch._C._autograd, "_top_saved_tensors_default_hooks", lambda ignore_tracing: None)
 
 
 def _address(g):
@@ -81,9 +79,11 @@ class SarEntropy(torch.autograd.Function):
     @staticmethod
     def forward(ctx, phi, rc, ha, rc_dtype: int, ws: Workspace, keep: bool = False):
         n_rg, n_az = rc.shape[0], rc.shape[1]
-        phi_c = phi.detach().contiguous()
+        phi_c = phi.detach()
+        if not phi_c.is_contiguous():
+            phi_c = phi_c.contiguous()
         ctx.rc, ctx.ha, ctx.rc_dtype, ctx.ws = rc, ha, rc_dtype, ws
-        keep = keep and ws.arith == B.ARITH_F32 and n_rg > 0 and not _saved_tensor_hooks()
+        keep = keep and ws.arith == B.ARITH_F32 and n_rg > 0 and _saved_tensor_hooks(False) is None
         versions = _versions(rc, ha) if keep else None
         if versions is not None:
             size = B.sar_autofocus_state_bytes(n_az, n_rg)
