@@ -820,6 +820,10 @@ LaunchSetup setup_kernel(K kern, int threads, size_t smem) {
 // Pure FP16 rows, 4096 points, 256 lines 12.4 -> 8.9 us, 4096 lines 61.7 -> 57.4;
 // adaptive exponents, 4096 lines 43.3 -> 41.9.
 // `chained` is false where it measured slower (launch_tc_kernel, uneven.cu).
+// Filter lines of 2048 or 4096 points with FP16 results, 257 to 380 CTAs, lose up
+// to 9 % when the same call runs back to back (the waiting CTAs crowd some SMs:
+// 8.5 -> 9.4 us); unchained, their turned and FP32 forms lose more (4096 points,
+// 160 lines: 11.2 -> 12.4 and 8.4 -> 10.1 us).
 // `cluster`: CTAs per thread-block cluster.
 template <class K, class... A>
 cudaError_t launch_chained(K kern, long long grid, int threads, size_t smem, int cluster, bool chained,

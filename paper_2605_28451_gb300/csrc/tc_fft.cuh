@@ -401,7 +401,9 @@ __device__ __forceinline__ void tc_cta_teardown(bool ok, unsigned char* smem, ui
 // bounds it is that chain of passes (barrier, MMA, accumulator read, twiddles,
 // store), not DRAM: one barrier a pass instead of two took 32768 lines from
 // .2093 to .2054 ms and the compression of 8192 lines from .1129 to .1092, the
-// early loads the former to .2035 (5.28 TB/s).
+// early loads the former to .2035.  The branch around the last stores (tc_valid)
+// keeps their addresses out of the passes before, which ends the spills: 65536
+// lines .3873 -> .3776 ms (5.69 TB/s).
 template <int MODE, class TIn, class TOut = __half2>
 __global__ void __launch_bounds__(tc::kThreads, tc::kCtasPerSm) fft_tc_kernel(const RowArgs a) {
   using namespace tc;
